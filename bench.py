@@ -89,14 +89,14 @@ def alu_roofline(updates: float, seconds: float, eq: str, dtype: str) -> dict:
 NCU_TRAFFIC = {
     # dram__bytes_read.sum + dram__bytes_write.sum of the whole 10^4-step solve in
     # one dataflow launch: a one-pass capture of the benchmark's own timed launch
-    "swept_batch_kernel<double,KS> n=1024 threads=256": {"src": "3b6f26f5347ef8b7", "bytes_per_launch": 11734272},
+    "swept_batch_kernel<double,KS> n=1024 threads=256": {"src": "36cee9459e5c736b", "bytes_per_launch": 11540000},
 }
 # Issue-slot use of the batched FP32 launch from one ncu capture (the 4096
 # instances of the batched workload, every node width 2048 fitted to N): warp
 # instructions issued over 4 per SM per cycle, keyed like the traffic record
 # and reported when the timed batch runs that width.
-NCU_ISSUE_FP32_BATCH = {"src": "3b6f26f5347ef8b7", "width": 2048, "issue_frac": 0.70, "issue_active": 0.703,
-                        "fma_pipe": 0.402}
+NCU_ISSUE_FP32_BATCH = {"src": "36cee9459e5c736b", "width": 2048, "issue_frac": 0.699, "issue_active": 0.701,
+                        "fma_pipe": 0.401}
 KERNEL_OF_LAUNCH = {"per_phase": "swept_phase_kernel", "graph": "swept_phase_kernel",
                     "persistent": "swept_batch_kernel", "auto": "swept_batch_kernel"}
 

@@ -33,8 +33,10 @@ __device__ __forceinline__ R bc_load(const R* arr, int64_t g, int64_t N, int bc,
 template <typename R, int EQ>
 __global__ void __launch_bounds__(256) classic_kernel(const R* __restrict__ src, const R* base,
                                                       R* out, int64_t N, int stage, int bc,
-                                                      Coefs<R> c)
+                                                      Coefs<R> cp)
 {
+    const Coefs<R> c = lane_coefs<R, EQ>(cp);
+    const Units<R> ku = make_units<R, EQ>();
     constexpr int RAD = EQ == HEAT ? 1 : 2;
     constexpr int NV = EQ == EULER ? 3 : 1;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -58,7 +60,7 @@ __global__ void __launch_bounds__(256) classic_kernel(const R* __restrict__ src,
         const int GW = TILE + 1;
         R* Cc = G + 3 * GW;         // cached (u, e, sqrt(rho)) of staged cell s at Cc[k SW + s]
         for (int s = threadIdx.x; s < SW; s += T) {
-            P[s] = euler_cell(sm[s], sm[SW + s], sm[2 * SW + s], c.gm1, Cc[s], Cc[SW + s], Cc[2 * SW + s]);
+            P[s] = euler_cell(sm[s], sm[SW + s], sm[2 * SW + s], c.gm1, Cc[s], Cc[SW + s], Cc[2 * SW + s], ku);
         }
         __syncthreads();
         for (int l = threadIdx.x; l < GW; l += T) {
@@ -69,20 +71,20 @@ __global__ void __launch_bounds__(256) classic_kernel(const R* __restrict__ src,
             const R ca[3] = {Cc[sb - 1], Cc[SW + sb - 1], Cc[2 * SW + sb - 1]};
             const R cb[3] = {Cc[sb], Cc[SW + sb], Cc[2 * SW + sb]};
             R g3[3];
-            euler_interface_cached(qa, qb, P[sb - 2], P[sb - 1], P[sb], P[sb + 1], ca, cb, c.gm1, c.ggm1, g3);
+            euler_interface_cached(qa, qb, P[sb - 2], P[sb - 1], P[sb], P[sb + 1], ca, cb, c.gm1, c.ggm1, g3, ku);
             G[l] = g3[0];
             G[GW + l] = g3[1];
             G[2 * GW + l] = g3[2];
         }
         __syncthreads();
-        const R kh = c.kh[stage];
+        const R kh = stage ? c.kh[1] : c.kh[0];
         for (int l = threadIdx.x; l < TILE; l += T) {
             const int64_t i = t0 + l;
             if (i >= N) break;
 #pragma unroll
             for (int v = 0; v < 3; ++v) {
                 const R b = stage == 0 ? sm[v * SW + RAD + l] : base[v * N + i];   // predictor: base = source
-                out[v * N + i] = euler_update(G[v * GW + l + 1], G[v * GW + l], b, kh);
+                out[v * N + i] = euler_update(G[v * GW + l + 1], G[v * GW + l], b, kh, ku);
             }
         }
     } else {
@@ -91,11 +93,12 @@ __global__ void __launch_bounds__(256) classic_kernel(const R* __restrict__ src,
             if (i >= N) break;
             const int s = RAD + l;
             if constexpr (EQ == HEAT) {
-                out[i] = heat_point(sm[s - 1], sm[s], sm[s + 1], c.fo);
+                out[i] = heat_point(sm[s - 1], sm[s], sm[s + 1], c.fo, ku);
             } else {
                 const R b = stage == 0 ? sm[s] : base[i];   // predictor: base = source
                 out[i] = ks_point(sm[s - 2], sm[s - 1], sm[s], sm[s + 1], sm[s + 2], b,
-                                  c.a1[stage], c.a4[stage], c.beta[stage], c.gam[stage]);
+                                  stage ? c.a1[1] : c.a1[0], stage ? c.a4[1] : c.a4[0],
+                                  stage ? c.beta[1] : c.beta[0], stage ? c.gam[1] : c.gam[0], ku);
             }
         }
     }
@@ -145,8 +148,10 @@ __device__ __forceinline__ void vec_load_bc(const R* arr, int64_t vi, int64_t nv
 template <typename R, int EQ, int U>
 __global__ void __launch_bounds__(256) classic_vec_kernel(const R* __restrict__ src, const R* base,
                                                           R* out, int64_t N, int stage, int bc,
-                                                          Coefs<R> c)
+                                                          Coefs<R> cp)
 {
+    const Coefs<R> c = lane_coefs<R, EQ>(cp);
+    const Units<R> ku = make_units<R, EQ>();
     constexpr int VW = Vec16<R>::W;
     using T = typename Vec16<R>::T;
     const int lane = threadIdx.x & 31;
@@ -175,7 +180,7 @@ __global__ void __launch_bounds__(256) classic_vec_kernel(const R* __restrict__ 
         R o[VW];
         if constexpr (EQ == HEAT) {
 #pragma unroll
-            for (int i = 0; i < VW; ++i) o[i] = heat_point(a[VW + i - 1], a[VW + i], a[VW + i + 1], c.fo);
+            for (int i = 0; i < VW; ++i) o[i] = heat_point(a[VW + i - 1], a[VW + i], a[VW + i + 1], c.fo, ku);
         } else {
             R b[VW];
             if (stage == 0) {   // predictor: the base is the source vector itself
@@ -187,7 +192,8 @@ __global__ void __launch_bounds__(256) classic_vec_kernel(const R* __restrict__ 
 #pragma unroll
             for (int i = 0; i < VW; ++i)
                 o[i] = ks_point(a[VW + i - 2], a[VW + i - 1], a[VW + i], a[VW + i + 1], a[VW + i + 2], b[i],
-                                c.a1[stage], c.a4[stage], c.beta[stage], c.gam[stage]);
+                                stage ? c.a1[1] : c.a1[0], stage ? c.a4[1] : c.a4[0],
+                                stage ? c.beta[1] : c.beta[0], stage ? c.gam[1] : c.gam[0], ku);
         }
         reinterpret_cast<T*>(out)[vi] = *reinterpret_cast<const T*>(o);
     }

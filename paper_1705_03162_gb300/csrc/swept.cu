@@ -183,19 +183,20 @@ __device__ __forceinline__ void window_store(R* A, R* B, const R* row0, const R*
 // tsh: log2 of the block size when that is a power of two, else -1.
 template <typename R, int EQ, int STAGE>
 __device__ __forceinline__ R run_point(const R (&v)[2 * Shape<EQ>::RAD + 1], const R* dst, int q,
-                                       const Coefs<R>& c)
+                                       const Coefs<R>& c, const Units<R>& k)
 {
     if constexpr (EQ == HEAT) {
-        return heat_point(v[0], v[1], v[2], c.fo);
+        return heat_point(v[0], v[1], v[2], c.fo, k);
     } else {
         const R base = STAGE == 0 ? v[2] : dst[q];
         return ks_point(v[0], v[1], v[2], v[3], v[4], base, c.a1[STAGE], c.a4[STAGE], c.beta[STAGE],
-                        c.gam[STAGE]);
+                        c.gam[STAGE], k);
     }
 }
 
 template <typename R, int EQ, int STAGE>
-__device__ __forceinline__ void level_runs(const R* src, R* dst, int lo, int cnt, int tsh, const Coefs<R>& c)
+__device__ __forceinline__ void level_runs(const R* src, R* dst, int lo, int cnt, int tsh, const Coefs<R>& c,
+                                           const Units<R>& ku)
 {
     constexpr int RAD = Shape<EQ>::RAD, U = 2 * RAD + 1;
     const int T = blockDim.x, m = cnt + T - 1;
@@ -218,17 +219,17 @@ __device__ __forceinline__ void level_runs(const R* src, R* dst, int lo, int cnt
         for (int u = 0; u < U; ++u) {
             v[U - 1] = nv[u];
             if constexpr (EQ == HEAT)
-                dst[q + u] = heat_point(v[0], v[1], v[2], c.fo);
+                dst[q + u] = heat_point(v[0], v[1], v[2], c.fo, ku);
             else
                 dst[q + u] = ks_point(v[0], v[1], v[2], v[3], v[4], STAGE == 0 ? v[2] : base[u], c.a1[STAGE],
-                                      c.a4[STAGE], c.beta[STAGE], c.gam[STAGE]);
+                                      c.a4[STAGE], c.beta[STAGE], c.gam[STAGE], ku);
 #pragma unroll
             for (int k = 0; k < U - 1; ++k) v[k] = v[k + 1];
         }
     }
     for (; q < end; ++q) {
         v[U - 1] = src[q + RAD];
-        dst[q] = run_point<R, EQ, STAGE>(v, dst, q, c);
+        dst[q] = run_point<R, EQ, STAGE>(v, dst, q, c, ku);
 #pragma unroll
         for (int k = 0; k < U - 1; ++k) v[k] = v[k + 1];
     }
@@ -243,7 +244,7 @@ __device__ __forceinline__ void level_runs(const R* src, R* dst, int lo, int cnt
 template <typename R, int EQ, bool RUNS>
 __device__ __forceinline__ void tile_levels(R* row0, R* row1, R* P, R* G, int nk, int H, int j_lo,
                                             int j_hi, int64_t g0, int64_t N, bool wall, int bc,
-                                            const Coefs<R>& c)
+                                            const Coefs<R>& c, const Units<R>& ku)
 {
     constexpr int RAD = Shape<EQ>::RAD;
     const int W = window_width(nk, RAD);
@@ -260,7 +261,7 @@ __device__ __forceinline__ void tile_levels(R* row0, R* row1, R* P, R* G, int nk
         const int stage = (EQ == HEAT) ? 0 : ((j & 1) ? 0 : 1);
         if constexpr (EQ == HEAT) {
             if (RUNS && sizeof(R) == 4 && !wall) {
-                level_runs<R, EQ, 0>(src, dst, lo, cnt, tsh, c);
+                level_runs<R, EQ, 0>(src, dst, lo, cnt, tsh, c, ku);
                 __syncthreads();
                 continue;
             }
@@ -274,14 +275,14 @@ __device__ __forceinline__ void tile_levels(R* row0, R* row1, R* P, R* G, int nk
                     tm = src[q - 1];
                     tp = src[q + 1];
                 }
-                dst[q] = heat_point(tm, src[q], tp, c.fo);
+                dst[q] = heat_point(tm, src[q], tp, c.fo, ku);
             }
         } else if constexpr (EQ == KS) {
             // KS problems are periodic: the window is already wrapped.  (The
             // stage picks by value: c may be a copy in registers.)
             if constexpr (RUNS && sizeof(R) == 4) {
-                if (stage) level_runs<R, EQ, 1>(src, dst, lo, cnt, tsh, c);
-                else level_runs<R, EQ, 0>(src, dst, lo, cnt, tsh, c);
+                if (stage) level_runs<R, EQ, 1>(src, dst, lo, cnt, tsh, c, ku);
+                else level_runs<R, EQ, 0>(src, dst, lo, cnt, tsh, c, ku);
                 __syncthreads();
                 continue;
             }
@@ -291,10 +292,10 @@ __device__ __forceinline__ void tile_levels(R* row0, R* row1, R* P, R* G, int nk
                 const int q = lo + t;
                 const R base = stage == 0 ? src[q] : row0[q];
                 dst[q] = ks_point(src[q - 2], src[q - 1], src[q], src[q + 1], src[q + 2], base, a1,
-                                  a4, beta, gam);
+                                  a4, beta, gam, ku);
             }
         } else {
-            const R kh = c.kh[stage];
+            const R kh = stage ? c.kh[1] : c.kh[0];
             // pressures (and the cell values euler_cell caches) of cells
             // [lo-2, hi+2), interfaces [lo, hi], then cells
             const int GW = W + 1;
@@ -318,11 +319,12 @@ __device__ __forceinline__ void tile_levels(R* row0, R* row1, R* P, R* G, int nk
                 Gh[2 + threadIdx.x] = gs[1];
                 Gh[4 + threadIdx.x] = gs[2];
                 Gh[6 + threadIdx.x] = euler_cell(gs[0], gs[1], gs[2], c.gm1, Gh[8 + threadIdx.x],
-                                                 Gh[10 + threadIdx.x], Gh[12 + threadIdx.x]);
+                                                 Gh[10 + threadIdx.x], Gh[12 + threadIdx.x], ku);
             }
             for (int t = threadIdx.x; t < cnt + 4; t += T) {
                 const int s = lo - 2 + t;
-                P[s] = euler_cell(src[s], src[W + s], src[2 * W + s], c.gm1, Cc[s], Cc[W + s], Cc[2 * W + s]);
+                P[s] = euler_cell(src[s], src[W + s], src[2 * W + s], c.gm1, Cc[s], Cc[W + s], Cc[2 * W + s],
+                                  ku);
             }
             __syncthreads();
             for (int t = threadIdx.x; t <= cnt; t += T) {
@@ -354,7 +356,8 @@ __device__ __forceinline__ void tile_levels(R* row0, R* row1, R* P, R* G, int nk
                         }
                     }
                     R g3[3];
-                    euler_interface_cached(q[0], q[1], p[0], p[1], p[2], p[3], cc[0], cc[1], c.gm1, c.ggm1, g3);
+                    euler_interface_cached(q[0], q[1], p[0], p[1], p[2], p[3], cc[0], cc[1], c.gm1, c.ggm1, g3,
+                                           ku);
                     R* o = rep ? Gx : G + sb;
                     const int os = rep ? 1 : GW;
                     o[0] = g3[0];
@@ -370,7 +373,7 @@ __device__ __forceinline__ void tile_levels(R* row0, R* row1, R* P, R* G, int nk
                 for (int v = 0; v < 3; ++v) {
                     const R base = stage == 0 ? src[v * W + q] : row0[v * W + q];
                     const R gp = last ? Gx[v] : G[v * GW + q + 1];
-                    dst[v * W + q] = euler_update(gp, G[v * GW + q], base, kh);
+                    dst[v * W + q] = euler_update(gp, G[v * GW + q], base, kh, ku);
                 }
             }
         }
@@ -385,7 +388,7 @@ __device__ __forceinline__ void tile_levels(R* row0, R* row1, R* P, R* G, int nk
 template <typename R, int EQ, int P, bool ODD>
 __device__ __forceinline__ void reg_level(const R (&src)[P], R (&dst)[P], R* xb, const R (&hl)[Shape<EQ>::RAD],
                                           const R (&hr)[Shape<EQ>::RAD], int j, int H, int cs, int s0,
-                                          const Coefs<R>& c)
+                                          const Coefs<R>& c, const Units<R>& ku)
 {
     constexpr int RAD = Shape<EQ>::RAD;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -427,11 +430,11 @@ __device__ __forceinline__ void reg_level(const R (&src)[P], R (&dst)[P], R* xb,
         };
         R v;
         if constexpr (EQ == HEAT) {
-            v = heat_point(at(-1), at(0), at(1), c.fo);
+            v = heat_point(at(-1), at(0), at(1), c.fo, ku);
         } else {
             const R base = ODD ? src[i] : dst[i];
             v = ks_point(at(-2), at(-1), at(0), at(1), at(2), base, c.a1[stage], c.a4[stage], c.beta[stage],
-                         c.gam[stage]);
+                         c.gam[stage], ku);
         }
         const int q = s0 + i;
         dst[i] = (q >= lo && q < hi) ? v : dst[i];
@@ -447,7 +450,7 @@ __device__ __forceinline__ void reg_level(const R (&src)[P], R (&dst)[P], R* xb,
 // memory at the end.  j_lo is always odd (H + 1 or 1, H even).
 template <typename R, int EQ, int P>
 __device__ __forceinline__ void tile_levels_reg(R* row0, R* row1, R* xb, int n, int H, int j_lo, int j_hi,
-                                                const Coefs<R>& c)
+                                                const Coefs<R>& c, const Units<R>& ku)
 {
     constexpr int RAD = Shape<EQ>::RAD;
     static_assert(P >= RAD, "a thread must own at least rad slots");
@@ -466,8 +469,8 @@ __device__ __forceinline__ void tile_levels_reg(R* row0, R* row1, R* xb, int n, 
         hr[k] = row1[n + RAD + k];
     }
     for (int j = j_lo; j <= j_hi; j += 2) {
-        reg_level<R, EQ, P, true>(r0, r1, xb, hl, hr, j, H, cs, s0, c);
-        if (j + 1 <= j_hi) reg_level<R, EQ, P, false>(r1, r0, xb, hl, hr, j + 1, H, cs, s0, c);
+        reg_level<R, EQ, P, true>(r0, r1, xb, hl, hr, j, H, cs, s0, c, ku);
+        if (j + 1 <= j_hi) reg_level<R, EQ, P, false>(r1, r0, xb, hl, hr, j + 1, H, cs, s0, c, ku);
     }
 #pragma unroll
     for (int i = 0; i < P; ++i) {
@@ -519,24 +522,27 @@ __device__ __forceinline__ bool node_near_wall(int bc, int k, int K)
 // otherwise in shared memory.
 template <typename R, int EQ, int PR>
 __device__ __forceinline__ void run_levels(R* row0, R* row1, R* P, R* G, int n, int nk, int H, int j_lo,
-                                           int j_hi, int64_t g0, int64_t N, bool wall, int bc, const Coefs<R>& c)
+                                           int j_hi, int64_t g0, int64_t N, bool wall, int bc, const Coefs<R>& c,
+                                           const Units<R>& ku)
 {
     if constexpr (PR > 0 && EQ != EULER) {
         if (!wall && nk == n) {
-            tile_levels_reg<R, EQ, PR>(row0, row1, P, n, H, j_lo, j_hi, c);
+            tile_levels_reg<R, EQ, PR>(row0, row1, P, n, H, j_lo, j_hi, c, ku);
             return;
         }
     }
     // (tiles of the register-blocked kernels that fall back here, wider or
     // next to a wall, keep the strided loop: fewer registers for the kernel)
-    tile_levels<R, EQ, PR == 0>(row0, row1, P, G, nk, H, j_lo, j_hi, g0, N, wall, bc, c);
+    tile_levels<R, EQ, PR == 0>(row0, row1, P, G, nk, H, j_lo, j_hi, g0, N, wall, bc, c, ku);
 }
 
 template <typename R, int EQ, int PR>
 __global__ void __launch_bounds__(EQ == EULER ? 256 : 1024) swept_phase_kernel(R* A, R* B, PhaseGeom g, int bc,
-                                                           Coefs<R> c)
+                                                           Coefs<R> cp)
 {
     constexpr int RAD = Shape<EQ>::RAD;
+    const Coefs<R> c = lane_coefs<R, EQ>(cp);
+    const Units<R> ku = make_units<R, EQ>();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int k = blockIdx.x;
     int64_t g0;
@@ -548,7 +554,7 @@ __global__ void __launch_bounds__(EQ == EULER ? 256 : 1024) swept_phase_kernel(R
     window_load<R, EQ, false>(A, B, row0, row1, nk, g0, g.N, need_b);
     __syncthreads();
     run_levels<R, EQ, PR>(row0, row1, P, G, g.n, nk, g.H, g.j_lo, g.j_hi, g0, g.N,
-                          node_near_wall(bc, k, g.K), bc, c);
+                          node_near_wall(bc, k, g.K), bc, c, ku);
     window_store<R, EQ, false>(A, B, row0, row1, nk, g0, g.N);
 }
 
@@ -614,20 +620,10 @@ __device__ __forceinline__ void batch_item(const BatchInst<R>& in, int k, int64_
     R *row0, *row1, *P, *G;
     smem_rows<R, EQ>(smem_raw, nk, row0, row1, P, G);
     window_load<R, EQ, true>(in.A, in.B, row0, row1, nk, g0, in.N, j_lo <= H);
-    // heat / KS: the point-update coefficients in registers for all levels,
-    // rather than re-read from the instance table after every level barrier
-    Coefs<R> cr{};
-    if constexpr (EQ != EULER) {
-        cr.fo = in.c.fo;
-#pragma unroll
-        for (int s = 0; s < 2; ++s) {
-            cr.a1[s] = in.c.a1[s];
-            cr.a4[s] = in.c.a4[s];
-            cr.beta[s] = in.c.beta[s];
-            cr.gam[s] = in.c.gam[s];
-        }
-    }
-    const Coefs<R>& c = EQ != EULER ? cr : in.c;
+    // the point-update coefficients in registers for all levels, rather than
+    // re-read from the instance table after every level barrier
+    const Coefs<R> c = lane_coefs<R, EQ>(in.c);
+    const Units<R> ku = make_units<R, EQ>();
     __syncthreads();
     bool done = false;
     if constexpr (REG && EQ != EULER) {
@@ -635,12 +631,12 @@ __device__ __forceinline__ void batch_item(const BatchInst<R>& in, int k, int64_
         // evenly over the block; this instance's may not)
         done = !node_near_wall(in.bc, k, in.K) && nk == n && n % (int)blockDim.x == 0;
         if (done) switch (n / (int)blockDim.x) {
-        case 2: tile_levels_reg<R, EQ, 2>(row0, row1, P, n, H, j_lo, j_hi, c); break;
-        case 4: tile_levels_reg<R, EQ, 4>(row0, row1, P, n, H, j_lo, j_hi, c); break;
-        case 8: tile_levels_reg<R, EQ, 8>(row0, row1, P, n, H, j_lo, j_hi, c); break;
+        case 2: tile_levels_reg<R, EQ, 2>(row0, row1, P, n, H, j_lo, j_hi, c, ku); break;
+        case 4: tile_levels_reg<R, EQ, 4>(row0, row1, P, n, H, j_lo, j_hi, c, ku); break;
+        case 8: tile_levels_reg<R, EQ, 8>(row0, row1, P, n, H, j_lo, j_hi, c, ku); break;
         case 16:
             if constexpr (sizeof(R) == 4) {
-                tile_levels_reg<R, EQ, 16>(row0, row1, P, n, H, j_lo, j_hi, c);
+                tile_levels_reg<R, EQ, 16>(row0, row1, P, n, H, j_lo, j_hi, c, ku);
                 break;
             }
             done = false;
@@ -650,7 +646,7 @@ __device__ __forceinline__ void batch_item(const BatchInst<R>& in, int k, int64_
     }
     if (!done)
         run_levels<R, EQ, 0>(row0, row1, P, G, n, nk, H, j_lo, j_hi, g0, in.N, node_near_wall(in.bc, k, in.K),
-                             in.bc, c);
+                             in.bc, c, ku);
     window_store<R, EQ, true>(in.A, in.B, row0, row1, nk, g0, in.N);
 }
 
@@ -678,6 +674,8 @@ __device__ __forceinline__ void classic_item(const BatchInst<R>& in, int k, int6
 {
     constexpr int RAD = Shape<EQ>::RAD, NV = Shape<EQ>::NV;
     const int64_t N = in.N;
+    const Coefs<R> c = lane_coefs<R, EQ>(in.c);
+    const Units<R> ku = make_units<R, EQ>();
     // chunk k is [floor(kN/K), floor((k+1)N/K)), with kN split so that it
     // cannot overflow (N < 2^35, K < 2^30)
     const int64_t q = N / in.K, rem = N % in.K;
@@ -698,13 +696,15 @@ __device__ __forceinline__ void classic_item(const BatchInst<R>& in, int k, int6
     __syncthreads();
     if constexpr (EQ == HEAT) {
         for (int l = threadIdx.x; l < cnt; l += T)
-            __stcg(dst + x0 + l, heat_point(sm[l], sm[l + 1], sm[l + 2], in.c.fo));
+            __stcg(dst + x0 + l, heat_point(sm[l], sm[l + 1], sm[l + 2], c.fo, ku));
     } else if constexpr (EQ == KS) {
-        const R a1 = in.c.a1[stage], a4 = in.c.a4[stage], beta = in.c.beta[stage], gam = in.c.gam[stage];
+        const R a1 = stage ? c.a1[1] : c.a1[0], a4 = stage ? c.a4[1] : c.a4[0];
+        const R beta = stage ? c.beta[1] : c.beta[0], gam = stage ? c.gam[1] : c.gam[0];
         for (int l = threadIdx.x; l < cnt; l += T) {
             const int q = RAD + l;
             const R base = stage == 0 ? sm[q] : __ldcg(in.A + x0 + l);
-            __stcg(dst + x0 + l, ks_point(sm[q - 2], sm[q - 1], sm[q], sm[q + 1], sm[q + 2], base, a1, a4, beta, gam));
+            __stcg(dst + x0 + l,
+                   ks_point(sm[q - 2], sm[q - 1], sm[q], sm[q + 1], sm[q + 2], base, a1, a4, beta, gam, ku));
         }
     } else {
         R* P = sm + NV * W;   // pressure of every staged cell
@@ -712,7 +712,7 @@ __device__ __forceinline__ void classic_item(const BatchInst<R>& in, int k, int6
         const int GW = cnt + 1;
         R* Cc = G + 3 * GW;   // cached (u, e, sqrt(rho)) of staged cell s at Cc[k W + s]
         for (int s = threadIdx.x; s < W; s += T)
-            P[s] = euler_cell(sm[s], sm[W + s], sm[2 * W + s], in.c.gm1, Cc[s], Cc[W + s], Cc[2 * W + s]);
+            P[s] = euler_cell(sm[s], sm[W + s], sm[2 * W + s], c.gm1, Cc[s], Cc[W + s], Cc[2 * W + s], ku);
         __syncthreads();
         for (int l = threadIdx.x; l <= cnt; l += T) {
             const int sb = RAD + l;
@@ -721,18 +721,18 @@ __device__ __forceinline__ void classic_item(const BatchInst<R>& in, int k, int6
             const R ca[3] = {Cc[sb - 1], Cc[W + sb - 1], Cc[2 * W + sb - 1]};
             const R cb[3] = {Cc[sb], Cc[W + sb], Cc[2 * W + sb]};
             R g3[3];
-            euler_interface_cached(qa, qb, P[sb - 2], P[sb - 1], P[sb], P[sb + 1], ca, cb, in.c.gm1, in.c.ggm1, g3);
+            euler_interface_cached(qa, qb, P[sb - 2], P[sb - 1], P[sb], P[sb + 1], ca, cb, c.gm1, c.ggm1, g3, ku);
             G[l] = g3[0];
             G[GW + l] = g3[1];
             G[2 * GW + l] = g3[2];
         }
         __syncthreads();
-        const R kh = in.c.kh[stage];
+        const R kh = stage ? c.kh[1] : c.kh[0];
         for (int l = threadIdx.x; l < cnt; l += T) {
 #pragma unroll
             for (int v = 0; v < 3; ++v) {
                 const R base = stage == 0 ? sm[v * W + RAD + l] : __ldcg(in.A + v * N + x0 + l);
-                __stcg(dst + v * N + x0 + l, euler_update(G[v * GW + l + 1], G[v * GW + l], base, kh));
+                __stcg(dst + v * N + x0 + l, euler_update(G[v * GW + l + 1], G[v * GW + l], base, kh, ku));
             }
         }
     }
