@@ -89,9 +89,18 @@ typedef struct {
 
 /* How swp_advance_ex runs the swept scheme. */
 typedef enum {
-    SWP_LAUNCH_AUTO = 0,        /* library choice, from measurement, with
-                                   the default width: for periodic heat and
-                                   KS with N a multiple of 32, CLUSTER up to
+    SWP_LAUNCH_AUTO = 0,        /* library choice, from measurement.  With the
+                                   default width and block size, heat and KS
+                                   run in one launch that keeps the grid on
+                                   chip (halo tiles in registers, exchanged
+                                   between co-resident blocks) where that is
+                                   the faster form: in FP64 up to 2^17 points,
+                                   beyond that heat up to about 10^6; in FP32
+                                   up to about 2*10^6, and in tiles of the same
+                                   kind, a launch per some ten levels, above.
+                                   Otherwise (wider FP64 grids, Euler, a given
+                                   width, a stream under capture): periodic heat
+                                   and KS with N a multiple of 32, CLUSTER up to
                                    N = 2048 (FP64) or 4096 (FP32), then
                                    REGISTER up to 2^15 for FP64 heat, 2^14
                                    for FP64 KS, 2^18 for FP32 heat, 2^17 for
@@ -169,7 +178,10 @@ swp_status swp_write(swp_problem* p, const void* src, size_t src_bytes, int src_
  * the state is complete afterwards (Section 4.2: output only at closing
  * triangles); a final partial half-cycle is closed exactly.
  * Asynchronous on the problem's stream.  SWP_ETIMEOUT reports a persistent
- * launch whose bounded neighbour wait gave up (the state is then invalid).
+ * or on-chip launch whose bounded neighbour wait gave up (the state is then
+ * invalid).  An on-chip launch's halo words take at most 4 state sizes of
+ * device memory (a few MB at most), allocated by the first such advance and not
+ * counted against swp_set_memory_budget.
  * Each such wait gives up after 2 s of device global time, or after the
  * number of nanoseconds (1 to 10^12) in the environment variable
  * SWP_WAIT_LIMIT_NS, read once per process: raise it to run persistent
@@ -367,14 +379,14 @@ swp_status swp_server_stats(swp_server* s, swp_server_statistics* out);
 /* Finish admitted work, fail unadmitted requests, stop the thread, free all. */
 swp_status swp_server_destroy(swp_server* s);
 
-/* Fault-injection hook for tests of the persistent launch's bounded waits.
- * withhold != 0 makes every neighbour wait of later SWP_LAUNCH_PERSISTENT
- * advances of this problem wait for a flag value no node ever publishes, so
+/* Fault-injection hook for tests of the bounded waits of persistent and on-chip
+ * launches.  withhold != 0 makes every neighbour wait of later
+ * SWP_LAUNCH_PERSISTENT and on-chip advances of this problem wait for a flag value no node ever publishes, so
  * each wait gives up after wait_limit_ns nanoseconds (device global timer),
  * the kernel returns without computing, and the next swp_synchronize /
  * swp_read reports SWP_ETIMEOUT (the state is then invalid).  withhold = 0
  * restores normal waits; wait_limit_ns (in (0, 1e10]) bounds every wait of
- * later persistent advances either way (default 2 s).  Nothing faults, traps
+ * those advances either way (default 2 s).  Nothing faults, traps
  * or hangs.  The paper has no counterpart: its nodes synchronise only at
  * kernel boundaries (Section 3). */
 swp_status swp_debug_withhold_flags(swp_problem* p, int withhold, int64_t wait_limit_ns);

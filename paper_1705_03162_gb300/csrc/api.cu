@@ -19,6 +19,7 @@
 
 #include "../../include/swept.h"
 #include "launch.h"
+#include "resident.h"
 
 using namespace swp;
 
@@ -51,6 +52,13 @@ struct swp_problem {
     };
     std::vector<Graph> graphs;
     cudaStream_t capture_stream = nullptr;
+    // resident launch: its shape (K = 0: none for this N), the words its blocks
+    // exchange halos through, and the sequence number of the next exchange
+    bool shape_known = false;
+    ResidentShape shape;
+    uint64_t* words = nullptr;
+    int* resident_status = nullptr;   // status word of resident launches, once one has run
+    uint32_t seq = 1;
 };
 
 namespace {
@@ -394,17 +402,104 @@ swp_status run_swept_persistent(swp_problem* p, const SweptPlan& s, int threads)
     return persistent_via_batch(p, s, threads);
 }
 
+// A test hook makes every wait of a launch wait for what is never published.
+uint32_t withheld_offset(const swp_problem* p) { return p->inject_withheld_flags ? (1u << 30) : 0u; }
+
+// The resident form of the advance (resident.cu), where N has a shape for it.
+// Returns false (nothing done) when it has none, when the words cannot be allocated, or when
+// the stream is being captured: the sequence numbers are launch arguments, so
+// a replayed launch would accept the previous replay's words.
+template <typename R>
+bool run_swept_resident(swp_problem* p, int64_t steps, swp_status* st)
+{
+    if (!p->shape_known) {
+        p->shape_known = true;
+        if (!resident_plan(p->desc.eq, p->esize, p->N, p->sms, max_smem(p->device), &p->shape)) p->shape.K = 0;
+    }
+    if (p->shape.K == 0) return false;
+    const int64_t levels = steps * p->sub;
+    if (p->shape.waves > 1) {
+        const int64_t E = (int64_t)p->shape.L * p->shape.M;
+        for (int64_t done = 0; done < levels; done += E) {
+            const cudaError_t e = launch_swept_resident<R>(p->desc.eq, p->desc.bc, (const R*)p->rows[p->cur],
+                                                           (R*)p->rows[1 - p->cur], p->N, std::min(E, levels - done),
+                                                           p->shape, ResidentSync{}, coefs_of<R>(p), p->stream);
+            if (e != cudaSuccess) {
+                *st = cuda_fail(e, "tiled swept launch");
+                return true;
+            }
+            p->launches++;
+            p->cur = 1 - p->cur;
+        }
+        *st = SWP_OK;
+        return true;
+    }
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(p->stream, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    if (cap != cudaStreamCaptureStatusNone) return false;
+    const size_t bytes = 2 * sizeof(uint64_t) * resident_words(p->desc.eq, p->esize, p->N, p->shape);
+    cudaError_t e = cudaSuccess;
+    if (!p->words) {
+        // the words, and the status word behind them
+        e = cudaMalloc((void**)&p->words, bytes + sizeof(int));
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            p->words = nullptr;
+            return false;
+        }
+        e = cudaMemsetAsync(p->words, 0, bytes + sizeof(int), p->stream);
+        p->seq = 1;
+    }
+    const int64_t exchanges = resident_exchanges(p->shape, levels);
+    if (exchanges >= (int64_t)1 << 30) return false;
+    if (e == cudaSuccess && (uint64_t)p->seq + (uint64_t)exchanges >= (uint64_t)1 << 31) {
+        // sequence numbers start over on cleared words
+        e = cudaMemsetAsync(p->words, 0, bytes, p->stream);
+        p->seq = 1;
+    }
+    if (e != cudaSuccess) {
+        *st = cuda_fail(e, "resident workspace memset");
+        return true;
+    }
+    ResidentSync y;
+    y.words = p->words;
+    y.seq = p->seq;
+    y.wait_offset = withheld_offset(p);
+    y.wait_limit_ns = p->wait_limit_ns;
+    y.status = (int*)((char*)p->words + bytes);
+    e = launch_swept_resident<R>(p->desc.eq, p->desc.bc, (const R*)p->rows[p->cur], (R*)p->rows[1 - p->cur], p->N,
+                                 levels, p->shape, y, coefs_of<R>(p), p->stream);
+    if (e == cudaErrorCooperativeLaunchTooLarge) {   // the device cannot hold all blocks at once
+        cudaGetLastError();
+        p->shape.K = 0;
+        return false;
+    }
+    p->launches++;
+    p->resident_status = y.status;
+    p->seq += (uint32_t)exchanges;
+    *st = e == cudaSuccess ? SWP_OK : cuda_fail(e, "resident swept launch");
+    if (e == cudaSuccess) p->cur = 1 - p->cur;
+    return true;
+}
+
 // Reads the device status word of persistent launches (stream must be idle).
 swp_status check_device_status(swp_problem* p)
 {
-    if (!p->status) return SWP_OK;
-    int st = 0;
-    cudaError_t e = cudaMemcpy(&st, p->status, sizeof(int), cudaMemcpyDeviceToHost);
-    if (e != cudaSuccess) return cuda_fail(e, "status read");
-    if (st != 0) {
-        cudaMemset(p->status, 0, sizeof(int));
-        return fail(SWP_ETIMEOUT, "a node's bounded wait for its neighbours gave up; the state is invalid");
+    bool gave_up = false;
+    for (int* word : {p->status, p->resident_status}) {
+        if (!word) continue;
+        int st = 0;
+        cudaError_t e = cudaMemcpy(&st, word, sizeof(int), cudaMemcpyDeviceToHost);
+        if (e != cudaSuccess) return cuda_fail(e, "status read");
+        if (st != 0) {
+            cudaMemset(word, 0, sizeof(int));
+            gave_up = true;
+        }
     }
+    if (gave_up) return fail(SWP_ETIMEOUT, "a node's bounded wait for its neighbours gave up; the state is invalid");
     return SWP_OK;
 }
 
@@ -554,13 +649,18 @@ swp_status advance_typed(swp_problem* p, int64_t steps, const swp_advance_opts& 
         }
         return run_classic<R>(p, steps, o.threads);
     }
-    // AUTO for small periodic heat and KS, where phases are short and launch
+    // AUTO: the form that keeps the grid on chip where it is the faster one
+    // (resident_plan).  Otherwise, for small periodic heat and KS, where phases are short and launch
     // gaps and global round trips count (measured fastest on GB300): the
     // cluster form up to 2048 points in FP64 and 4096 in FP32 (heat FP32
     // N = 1024: 11.9 G point-updates/s against 2.2 for per-phase launches),
     // then the Register variant (graph) up to 2^15 (heat) and 2^14 (KS) in
     // FP64, and in FP32 for heat up to 2^18 (2^18: 566 against 528) and KS up
     // to 2^17; a cluster that cannot run falls through
+    if (o.launch == SWP_LAUNCH_AUTO && o.points_per_block == 0 && o.threads == 0) {
+        swp_status st = SWP_OK;
+        if (run_swept_resident<R>(p, steps, &st)) return st;
+    }
     if (o.launch == SWP_LAUNCH_AUTO && o.points_per_block == 0 && o.threads == 0 && p->desc.eq != SWP_EULER &&
         p->desc.bc == SWP_BC_PERIODIC && p->N % 32 == 0 && p->N >= 64) {
         const bool f32 = p->desc.dtype == SWP_F32;
@@ -791,6 +891,7 @@ swp_status swp_destroy(swp_problem* p)
     if (p->rows[0]) e = cudaFree(p->rows[0]);
     if (p->batch) swp_batch_destroy(p->batch);
     if (p->status) cudaFree(p->status);
+    if (p->words) cudaFree(p->words);
     for (auto& g : p->graphs) cudaGraphExecDestroy(g.exec);
     if (p->capture_stream) cudaStreamDestroy(p->capture_stream);
     g_in_use -= p->bytes;
@@ -1160,7 +1261,7 @@ swp_status persistent_via_batch(swp_problem* p, const SweptPlan& s, int threads)
     items[0].p_hi = s.n_phases;
     items[0].flip = false;   // the caller moves the state's row
     const int mode = p->desc.eq == SWP_EULER ? SWP_EULER : SWP_HEAT;
-    const uint32_t withhold = p->inject_withheld_flags ? (1u << 30) : 0u;
+    const uint32_t withhold = withheld_offset(p);
     // at most 768 threads (24 warps) per SM: with fewer nodes in flight each
     // finishes sooner and the phase chain advances faster (KS 2^20, 1024-point
     // nodes: 40.0 against 36.8 G upd/s with 5 blocks of 256 per SM)

@@ -1,0 +1,538 @@
+// Resident form of a single heat / KS advance: one launch, the state in
+// registers and shared memory from the first step to the last.
+//
+// The paper's nodes alternate an inverted and an upright triangle, so a
+// half-cycle of H levels takes 2H - 1 dependent levels; that is the shape that
+// needs no point twice, and it costs a grid that does not fill the GPU almost
+// two level latencies per level.  Here each block owns a contiguous part of
+// the grid and advances a tile of it with halos: a level leaves the outermost
+// rad points of the tile stale, and after h / rad levels the halos are
+// fetched again.  Every level of a tile is one level of progress; the price is
+// the halo points' work, which the geometry keeps to a few per cent where the
+// arithmetic counts and which is free where the chip would idle.
+//
+// Three scales:
+//  - a thread holds P consecutive points in registers; a level reads its rad
+//    neighbours on each side from the adjacent lanes by shuffle, and nothing
+//    is predicated (stale edge values are computed and ignored);
+//  - a warp advances L levels alone on 32 P points, of which 32 P - 2 rad L
+//    are then valid; they go through shared memory (double buffered, one
+//    barrier) and each warp reloads its points with fresh neighbours;
+//  - after M such rounds the block publishes its owned points that lie within
+//    h + 1 (h = rad L M) of its ends and fetches its halos from the neighbouring
+//    blocks.  Each published word carries the exchange's sequence number next
+//    to its data (8 bytes, stored and loaded as one access), so a reader polls
+//    the data itself: no flag, no fence, one trip through L2 each way.
+// The blocks wait on one another, so the launch is cooperative (all blocks
+// resident); every wait is bounded.  An FP32 grid that the chip does not hold
+// runs the same tiles without waits: a launch per L M levels, from one row to the
+// other.
+//
+// Both ends of the domain are index folds: periodic points wrap, and an
+// insulated end (u_{-k} = u_k, Appendix A) is the even extension, whose mirrored
+// points evolve with the same bits because the stencil's only sum of the two
+// neighbours commutes.
+//
+// Each point update is scheme.cuh's on the same operands as in the classic
+// scheme, so the bits are the same.
+//
+// What bounds it.  FP64: its pipe, at 66 clocks per warp-wide FMA; with one warp
+// per SM sub-partition the chain of a level (KS N = 1024: 550 of 670 clocks),
+// and the exchange of about 1450 clocks between blocks.  FP32: instruction
+// issue; 94 % of the instructions are the point updates' own (KS, 2000003
+// points; 67 % of issue slots used, the rest lost to register-bank limits of
+// three-operand FMAs).  Measured per advance against the forms that were the
+// default before (cluster, Register and Shared graphs, per-phase FP32):
+//   heat FP64 N = 1024, 4096 steps      1196 -> 610 us
+//   heat FP64 reflective 50001, 2000    1559 -> 807 us
+//   KS FP64 10007, 2000 steps           3224 -> 1575 us
+//   heat FP32 2^17, 4000 steps          1080 -> 178 us
+//   KS FP32 2000003, 1000 steps         3710 -> 1158 us
+#include <algorithm>
+
+#include "geometry.cuh"
+#include "resident.h"
+
+namespace swp {
+
+namespace {
+
+// Hard cap on polls of one wait, in case the global timer does not advance.
+constexpr uint32_t kMaxPolls = 1u << 26;
+
+__device__ __forceinline__ uint64_t global_ns()
+{
+    uint64_t t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    return t;
+}
+
+// Published words: data and sequence number in one 8-byte access (FP64: two
+// of them, each half of the value).
+template <typename R> struct Word;
+template <> struct Word<float> {
+    static constexpr int N64 = 1;
+    static __device__ __forceinline__ void put(uint64_t* p, float v, uint32_t seq)
+    {
+        const uint64_t w = (uint64_t)seq << 32 | __float_as_uint(v);
+        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
+    }
+    static __device__ __forceinline__ bool get(const uint64_t* p, float& v, uint32_t seq)
+    {
+        uint64_t w;
+        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
+        v = __uint_as_float((uint32_t)w);
+        return (uint32_t)(w >> 32) == seq;
+    }
+};
+template <> struct Word<double> {
+    static constexpr int N64 = 2;
+    static __device__ __forceinline__ void put(uint64_t* p, double v, uint32_t seq)
+    {
+        const uint64_t b = (uint64_t)__double_as_longlong(v), s = (uint64_t)seq << 32;
+        asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(s | (b & 0xffffffffu)),
+                     "l"(s | (b >> 32))
+                     : "memory");
+    }
+    static __device__ __forceinline__ bool get(const uint64_t* p, double& v, uint32_t seq)
+    {
+        uint64_t a, b;
+        asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+        v = __longlong_as_double((long long)((b << 32) | (a & 0xffffffffu)));
+        return (uint32_t)(a >> 32) == seq && (uint32_t)(b >> 32) == seq;
+    }
+};
+
+// Point of [0, N) that stands for point g of the extended line.
+__device__ __forceinline__ int64_t fold(int64_t g, int64_t N, int bc)
+{
+    const int64_t per = bc == PERIODIC ? N : 2 * (N - 1);
+    if (g < 0 || g >= per) {
+        g %= per;
+        if (g < 0) g += per;
+    }
+    return g < N ? g : per - g;
+}
+
+// FP32 runs of a multiple of 4 points move as 16-byte vectors.
+template <typename R, int P>
+constexpr bool kVector = sizeof(R) == 4 && P % 4 == 0;
+
+// Shared-memory index of tile slot s.  Lanes read runs of P slots, all lanes
+// at once, so the stride of the runs is padded to spread over the banks: vector
+// runs (FP32, P a multiple of 4) to an odd number of 16-byte vectors, even FP64
+// strides by a value after every 16.
+template <typename R, int P>
+__host__ __device__ __forceinline__ constexpr int slot_at(int s)
+{
+    if (kVector<R, P>) return (P / 4) % 2 ? s : s + s / P * 4;
+    if (sizeof(R) == 8 && P % 2 == 0) return s + (s >> 4);
+    return s;
+}
+
+template <typename R, int P>
+__device__ __forceinline__ void load_run(const R* buf, int s, R (&u)[P])
+{
+    if constexpr (kVector<R, P>) {
+#pragma unroll
+        for (int i = 0; i < P; i += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(buf + slot_at<R, P>(s) + i);   // s a multiple of P
+            u[i] = v.x;
+            u[i + 1] = v.y;
+            u[i + 2] = v.z;
+            u[i + 3] = v.w;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < P; ++i) u[i] = buf[slot_at<R, P>(s + i)];
+    }
+}
+
+// Store the points of a lane's run that are still valid: warp points
+// [edge, 32 P - edge).  Vector runs: edge is a multiple of P, so whole lanes.
+template <typename R, int P>
+__device__ __forceinline__ void store_run(R* buf, int s, const R (&u)[P], int lane, int edge)
+{
+    if constexpr (kVector<R, P>) {
+        if (lane * P >= edge && lane * P < 32 * P - edge) {
+#pragma unroll
+            for (int i = 0; i < P; i += 4)
+                *reinterpret_cast<float4*>(buf + slot_at<R, P>(s) + i) = make_float4(u[i], u[i + 1], u[i + 2], u[i + 3]);
+        }
+    } else {
+        const unsigned span = (unsigned)(32 * P - 2 * edge);
+        const int at = lane * P - edge;
+#pragma unroll
+        for (int i = 0; i < P; ++i)
+            if ((unsigned)(at + i) < span) buf[slot_at<R, P>(s + i)] = u[i];
+    }
+}
+
+// Values of the rad slots before (lo) and after (hi) this lane's run.
+template <typename R, int RAD, int P>
+__device__ __forceinline__ void run_edges(const R (&u)[P], R (&lo)[RAD], R (&hi)[RAD])
+{
+    if constexpr (P >= RAD) {
+#pragma unroll
+        for (int k = 0; k < RAD; ++k) {
+            lo[k] = __shfl_up_sync(0xffffffffu, u[P - RAD + k], 1);
+            hi[k] = __shfl_down_sync(0xffffffffu, u[k], 1);
+        }
+    } else {   // P == 1, RAD == 2
+        lo[0] = __shfl_up_sync(0xffffffffu, u[0], 2);
+        lo[1] = __shfl_up_sync(0xffffffffu, u[0], 1);
+        hi[0] = __shfl_down_sync(0xffffffffu, u[0], 1);
+        hi[1] = __shfl_down_sync(0xffffffffu, u[0], 2);
+    }
+}
+
+// One level of a lane's run: out = level after src (KS stage 1 with base
+// values from out).
+template <typename R, int EQ, int STAGE, int P>
+__device__ __forceinline__ void run_level(const R (&src)[P], R (&out)[P], const Coefs<R>& c,
+                                          const Units<R>& ku)
+{
+    constexpr int RAD = Shape<EQ>::RAD;
+    R lo[RAD], hi[RAD];
+    run_edges<R, RAD, P>(src, lo, hi);
+#pragma unroll
+    for (int i = 0; i < P; ++i) {
+        auto at = [&](int d) -> R {
+            const int q = i + d;
+            return q < 0 ? lo[RAD + q] : (q >= P ? hi[q - P] : src[q]);
+        };
+        if constexpr (EQ == HEAT)
+            out[i] = heat_point(at(-1), at(0), at(1), c.fo, ku);
+        else
+            out[i] = ks_point(at(-2), at(-1), at(0), at(1), at(2), STAGE == 0 ? src[i] : out[i], c.a1[STAGE],
+                              c.a4[STAGE], c.beta[STAGE], c.gam[STAGE], ku);
+    }
+}
+
+// `levels` levels of a lane's run (KS: an even number, whole timesteps).
+template <typename R, int EQ, int P>
+__device__ __forceinline__ void run_levels(R (&u)[P], int levels, const Coefs<R>& c, const Units<R>& ku)
+{
+    R v[P];
+#pragma unroll 1
+    for (int j = levels; j >= 2; j -= 2) {
+        run_level<R, EQ, 0, P>(u, v, c, ku);
+        run_level<R, EQ, 1, P>(v, u, c, ku);
+    }
+    if (EQ == HEAT && (levels & 1)) {
+        run_level<R, EQ, 0, P>(u, v, c, ku);
+#pragma unroll
+        for (int i = 0; i < P; ++i) u[i] = v[i];
+    }
+}
+
+template <typename R, int EQ, int P>
+__global__ void __launch_bounds__(512, sizeof(R) == 4 ? 1 : 0) swept_resident_kernel(const R* A, R* B, ResidentGeom g, Coefs<R> cp)
+{
+    const Coefs<R> c = lane_coefs<R, EQ>(cp);
+    const Units<R> ku = make_units<R, EQ>();
+    constexpr int RAD = Shape<EQ>::RAD;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    R* buf0 = reinterpret_cast<R*>(smem_raw);
+    R* buf1 = buf0 + g.buf_elems;
+    int* hoff = reinterpret_cast<int*>(buf1 + g.buf_elems);   // published word of each halo point
+    const int T = blockDim.x, tid = threadIdx.x, lane = tid & 31;
+    const int k = blockIdx.x, K = g.K, h = g.h;
+    const int64_t N = g.N;
+    const int64_t b0 = k * N / K;
+    const int own = (int)((k + 1) * N / K - b0);
+    const int edge = RAD * g.L;
+    // the lane's run starts at this tile slot; slot s is point b0 - h + s
+    const int s0 = (tid >> 5) * (32 * P - 2 * edge) + lane * P;
+    const int cap = g.cap, pub = g.pub;   // published points per block: all, or pub at each end
+    for (int s = tid; s < g.slots; s += T)
+        buf0[slot_at<R, P>(s)] = s < own + 2 * h ? A[fold(b0 - h + s, N, g.bc)] : R(0);
+    if (g.exchanges > 0) {
+        for (int e = tid; e < 2 * h; e += T) {
+            // 32-bit arithmetic: N K < 2^31 (resident_plan)
+            const int p = (int)fold(b0 - h + (e < h ? e : own + e), N, g.bc), n = (int)N;
+            const int o = ((p + 1) * K - 1) / n;   // the block that owns point p
+            const int ob = o * n / K;
+            const int on = (o + 1) * n / K - ob, at = p - ob;
+            hoff[e] = o * cap + (on <= 2 * pub || at < pub ? at : at - (on - 2 * pub));
+        }
+    }
+    __syncthreads();
+    R* cur = buf0;
+    R* nxt = buf1;
+    R u[P];
+    for (int64_t x = 0;; ++x) {
+        int left = x < g.exchanges ? g.E : g.last;   // levels until the next exchange, or the end
+        while (left > 0) {
+            const int n = min(left, g.L);
+            load_run<R, P>(cur, s0, u);
+            run_levels<R, EQ, P>(u, n, c, ku);
+            store_run<R, P>(nxt, s0, u, lane, edge);
+            __syncthreads();
+            R* t = cur;
+            cur = nxt;
+            nxt = t;
+            left -= n;
+        }
+        if (x >= g.exchanges) break;
+        const uint32_t seq = g.seq + (uint32_t)x + g.wait_offset;
+        uint64_t* words = g.words + (x & 1) * g.parity_words;
+        {
+            const int words_here = min(own, 2 * pub);
+            for (int i = tid; i < words_here; i += T) {
+                const int o = i < pub || own <= 2 * pub ? i : own - 2 * pub + i;
+                Word<R>::put(words + (int64_t)(k * cap + i) * Word<R>::N64, cur[slot_at<R, P>(h + o)],
+                             g.seq + (uint32_t)x);
+            }
+        }
+        int fail = 0;
+        for (int e = tid; e < 2 * h; e += T) {
+            const uint64_t* w = words + (int64_t)hoff[e] * Word<R>::N64;
+            R v;
+            uint32_t polls = 0;
+            uint64_t t0 = 0;
+            while (!Word<R>::get(w, v, seq)) {
+                if ((++polls & 255u) == 0) {
+                    const uint64_t now = global_ns();
+                    if (t0 == 0) t0 = now;
+                    if (*reinterpret_cast<volatile int*>(g.status) != 0 || now - t0 > g.wait_limit_ns ||
+                        polls > kMaxPolls) {
+                        atomicExch(g.status, 1);
+                        fail = 1;
+                        break;
+                    }
+                }
+            }
+            if (fail) break;
+            cur[slot_at<R, P>(e < h ? e : own + e)] = v;
+        }
+        if (__syncthreads_or(fail)) return;
+    }
+    for (int o = tid; o < own; o += T) B[b0 + o] = cur[slot_at<R, P>(h + o)];
+}
+
+// Kernel of (precision, equation, points per thread), or NULL.
+template <typename R, int EQ>
+const void* kernel_of(int P)
+{
+#define SWP_RESIDENT_P(p) \
+    case p: return (const void*)swept_resident_kernel<R, EQ, p>;
+    if constexpr (sizeof(R) == 8) {
+        switch (P) {
+            SWP_RESIDENT_P(1)
+            SWP_RESIDENT_P(2)
+            SWP_RESIDENT_P(3)
+            SWP_RESIDENT_P(4)
+            SWP_RESIDENT_P(5)
+            SWP_RESIDENT_P(6)
+            SWP_RESIDENT_P(7)
+            SWP_RESIDENT_P(8)
+            SWP_RESIDENT_P(9)
+            SWP_RESIDENT_P(10)
+            SWP_RESIDENT_P(11)
+            SWP_RESIDENT_P(12)
+            SWP_RESIDENT_P(13)
+            SWP_RESIDENT_P(14)
+            SWP_RESIDENT_P(15)
+            SWP_RESIDENT_P(16)
+        default: return nullptr;
+        }
+    } else {
+        switch (P) {
+            SWP_RESIDENT_P(1)
+            SWP_RESIDENT_P(2)
+            SWP_RESIDENT_P(4)
+            SWP_RESIDENT_P(8)
+            SWP_RESIDENT_P(12)
+            SWP_RESIDENT_P(16)
+            SWP_RESIDENT_P(20)
+            SWP_RESIDENT_P(24)
+            SWP_RESIDENT_P(28)
+            SWP_RESIDENT_P(32)
+        default: return nullptr;
+        }
+    }
+#undef SWP_RESIDENT_P
+}
+
+template <typename R>
+const void* kernel_of(int eq, int P)
+{
+    return eq == HEAT ? kernel_of<R, HEAT>(P) : kernel_of<R, KS>(P);
+}
+
+constexpr int kPoints64[] = {1, 2, 3, 4, 5, 6, 7, 8, 9, 10, 11, 12, 13, 14, 15, 16};
+constexpr int kPoints32[] = {1, 2, 4, 8, 12, 16, 20, 24, 28, 32};
+
+int slot_count(int P, int warps, int rad, int L) { return warps * (32 * P - 2 * rad * L) + 2 * rad * L; }
+
+// Elements of one shared-memory buffer (slot_at of the last slot, rounded up
+// to whole 16-byte vectors).
+int buffer_elems(int esize, int P, int slots)
+{
+    int e = slots;
+    if (esize == 4 && P % 8 == 0) e += (slots - 1) / P * 4;
+    if (esize == 8 && P % 2 == 0) e += (slots - 1) >> 4;
+    return (e + 3) / 4 * 4;
+}
+
+size_t smem_of(int esize, int P, int slots, int h)
+{
+    return 2 * (size_t)buffer_elems(esize, P, slots) * esize + sizeof(int) * 2 * (size_t)h;
+}
+
+}  // namespace
+
+namespace {
+
+// Estimated clocks (2.07 GHz) per level of a block of `warps` warps with P
+// points per thread that owns its tile's points, from a fit to 2294 measured
+// shapes (N from 2^10 to 2^21): the arithmetic of a level, the round through
+// shared memory every L levels (170 to 1000) and the exchange between blocks
+// every L M levels (1450 and the polls of its halo).  FP64 is its pipe's time
+// (66 clocks per warp-wide FMA) and a latency that a second warp per SM
+// sub-partition hides; FP32 is issue, at 1.1 (heat) and 1.36 (KS) slots per
+// operation, above the latency of a level's shuffles and chain.
+double level_clocks(int eq, int esize, int warps, int P, int L, int M, int h)
+{
+    const double ops = eq == HEAT ? 3.0 : 7.0, w = warps / 4;
+    double level;
+    if (esize == 8)
+        level = w * P * ops * 66.0 * (warps == 4 ? 1.06 : (warps == 8 ? 1.0 : 0.98)) + (warps == 4 ? 50.0 : 15.0);
+    else if (eq == HEAT)
+        level = std::max(57.0, 1.1 * w * P * ops + 35.0);
+    else
+        level = std::max(50.0 + 10.0 * std::min(P, 4), (warps == 4 ? 1.5 : 1.36) * w * P * ops + 25.0);
+    const double round = esize == 8 ? 170.0 + 12.0 * w * P : 130.0 + 6.0 * w * P;
+    const double exchange = M > 0 ? (1450.0 + 2.5 * h) / ((double)L * M) : 0.0;
+    return level + round / L + exchange;
+}
+
+// The best shape for blocks that own `own` points each.  Returns its clocks per
+// level, 0 when no tile holds them.
+double best_shape(int eq, int esize, int own, size_t max_smem, ResidentShape* out)
+{
+    const int rad = eq == HEAT ? 1 : 2;
+    const int* pts = esize == 8 ? kPoints64 : kPoints32;
+    const int npts = esize == 8 ? (int)(sizeof(kPoints64) / sizeof(int)) : (int)(sizeof(kPoints32) / sizeof(int));
+    double best = 0.0;
+    for (int warps = 4; warps <= 16; warps += 4)
+        for (int ip = 0; ip < npts; ++ip) {
+            const int P = pts[ip];
+            const bool vector = esize == 4 && P % 4 == 0;
+            for (int step = 1; step <= 8; ++step) {
+                // vector runs leave whole lanes stale
+                const int L = vector ? step * P / rad : 2 * step;
+                if (L & 1 || 2 * rad * L >= 32 * P - rad) continue;
+                const int slots = slot_count(P, warps, rad, L);
+                const int M = std::min(64, (slots - own) / (2 * rad * L));
+                if (M < 1) continue;
+                const int h = rad * L * M;
+                if (smem_of(esize, P, slots, h) > max_smem) continue;
+                const double cost = level_clocks(eq, esize, warps, P, L, M, h);
+                if (best == 0.0 || cost < best) {
+                    best = cost;
+                    out->P = P;
+                    out->warps = warps;
+                    out->L = L;
+                    out->M = M;
+                }
+            }
+        }
+    return best;
+}
+
+}  // namespace
+
+bool resident_plan(int eq, int esize, int64_t N, int sms, size_t max_smem, ResidentShape* out)
+{
+    *out = ResidentShape();
+    if (eq == EULER || N < 64 || sms < 1) return false;
+    const double ops = eq == HEAT ? 3.0 : 7.0;
+    // blocks of at least 16 points: with fewer the halos come from many blocks
+    const int K = (int)std::min<int64_t>(sms, std::max<int64_t>(1, N / 16));
+    if ((N + 1) * (K + 1) < (int64_t)1 << 31) {
+        const int own = (int)((N + K - 1) / K);
+        const double clocks = best_shape(eq, esize, own, max_smem, out);
+        // FP64 from 2^17 points: the swept dataflow launch spends about 700
+        // clocks per level above its points' pipe time (KS 2^17: 3760 against
+        // 3965 here, 2^20: 25530 against 25930; heat 2^17: 1995 against 1690)
+        if (clocks > 0.0 &&
+            (esize == 4 || N < ((int64_t)1 << 17) || clocks <= own / 128.0 * ops * 66.0 + 700.0)) {
+            out->K = K;
+            return true;
+        }
+    }
+    if (esize == 8) return false;
+    // FP32 beyond the chip: tiles of the same kind, a launch per exchange,
+    // whole waves of one block per SM.  (FP64 there is at its pipe's rate in
+    // the dataflow launch.)
+    const int64_t waves = (N + (int64_t)sms * 14000 - 1) / ((int64_t)sms * 14000);
+    const int64_t blocks = waves * sms;
+    if (blocks >= (int64_t)1 << 30) return false;
+    if (best_shape(eq, esize, (int)((N + blocks - 1) / blocks), max_smem, out) == 0.0) return false;
+    out->K = (int)blocks;
+    out->waves = (int)std::min<int64_t>(waves, 1 << 20);
+    return true;
+}
+
+size_t resident_words(int eq, int esize, int64_t N, const ResidentShape& s)
+{
+    const int rad = eq == HEAT ? 1 : 2;
+    const int own = (int)((N + s.K - 1) / s.K);
+    return (size_t)s.K * std::min(own, 2 * (rad * s.L * s.M + 1)) * (esize == 8 ? 2 : 1);
+}
+
+int64_t resident_exchanges(const ResidentShape& s, int64_t levels)
+{
+    const int64_t E = (int64_t)s.L * s.M;
+    return (levels + E - 1) / E - 1;
+}
+
+template <typename R>
+cudaError_t launch_swept_resident(int eq, int bc, const R* A, R* B, int64_t N, int64_t levels, const ResidentShape& s,
+                                  const ResidentSync& y, const Coefs<R>& c, cudaStream_t st)
+{
+    const int rad = eq == HEAT ? 1 : 2;
+    ResidentGeom g;
+    g.N = N;
+    g.K = s.K;
+    g.L = s.L;
+    g.E = s.L * s.M;
+    g.h = rad * g.E;
+    g.slots = slot_count(s.P, s.warps, rad, s.L);
+    const int own = (int)((N + s.K - 1) / s.K);
+    // the mirror image of a halo of h points reaches point h of the end block
+    g.pub = g.h + 1;
+    g.cap = std::min(own, 2 * g.pub);
+    g.exchanges = resident_exchanges(s, levels);
+    g.last = (int)(levels - g.exchanges * g.E);
+    g.bc = bc;
+    g.words = y.words;
+    g.parity_words = y.words ? (int64_t)resident_words(eq, (int)sizeof(R), N, s) : 0;
+    g.seq = y.seq;
+    g.wait_offset = y.wait_offset;
+    g.wait_limit_ns = y.wait_limit_ns;
+    g.status = y.status;
+    const size_t smem = smem_of((int)sizeof(R), s.P, g.slots, g.h);
+    g.buf_elems = buffer_elems((int)sizeof(R), s.P, g.slots);
+    const void* fn = kernel_of<R>(eq, s.P);
+    if (!fn) return cudaErrorInvalidDeviceFunction;
+    if (smem > 48 * 1024) {
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        if (e != cudaSuccess) return e;
+    }
+    void* args[] = {(void*)&A, (void*)&B, (void*)&g, (void*)&c};
+    const dim3 grid((unsigned)s.K), block((unsigned)(32 * s.warps));
+    return s.waves > 1 ? cudaLaunchKernel(fn, grid, block, args, smem, st)
+                       : cudaLaunchCooperativeKernel(fn, grid, block, args, smem, st);
+}
+
+template cudaError_t launch_swept_resident<double>(int, int, const double*, double*, int64_t, int64_t,
+                                                   const ResidentShape&, const ResidentSync&, const Coefs<double>&,
+                                                   cudaStream_t);
+template cudaError_t launch_swept_resident<float>(int, int, const float*, float*, int64_t, int64_t,
+                                                  const ResidentShape&, const ResidentSync&, const Coefs<float>&,
+                                                  cudaStream_t);
+
+}  // namespace swp

@@ -1,0 +1,52 @@
+// The resident form of a single heat / KS advance (resident.cu): launch
+// interface between the C-ABI layer (api.cu) and the kernel.  Internal header.
+#pragma once
+
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "scheme.cuh"
+
+namespace swp {
+
+// One cooperative launch of K blocks, each keeping its part of the grid on chip.
+struct ResidentShape {
+    int K = 0;        // blocks (0: N has no resident shape)
+    int waves = 1;    // > 1: more blocks than the chip holds; no exchanges, a launch per L M levels
+    int P = 0;        // points per thread
+    int warps = 0;    // warps per block
+    int L = 0, M = 0; // levels per warp round, rounds per exchange between blocks
+};
+// What a launch synchronises through: two sets of published words (one per
+// exchange parity), each word carrying the exchange's sequence number, which
+// no earlier launch on these words has used.
+struct ResidentSync {
+    uint64_t* words;
+    uint32_t seq;          // of the launch's first exchange
+    uint32_t wait_offset;  // 0; a test hook sets it so that no wait can succeed
+    uint64_t wait_limit_ns;
+    int* status;           // != 0: a wait gave up
+};
+struct ResidentGeom {
+    int64_t N;
+    int K, L, E, h;        // blocks, levels per round, levels per exchange, halo points per side
+    int slots, buf_elems;  // tile slots per block, elements of one shared-memory buffer
+    int pub, cap;          // points published at each end of a block, words per block
+    int bc, last;          // boundary; levels after the last exchange
+    int64_t exchanges, parity_words;
+    uint64_t* words;
+    uint32_t seq, wait_offset;
+    uint64_t wait_limit_ns;
+    int* status;
+};
+// The shape with the least estimated time per level, false when N does not fit.
+bool resident_plan(int eq, int esize, int64_t N, int sms, size_t max_smem, ResidentShape* out);
+// 8-byte words of one parity, and exchanges of an advance of `levels` levels.
+size_t resident_words(int eq, int esize, int64_t N, const ResidentShape& s);
+int64_t resident_exchanges(const ResidentShape& s, int64_t levels);
+// A -> B (the state ends in row B).
+template <typename R>
+cudaError_t launch_swept_resident(int eq, int bc, const R* A, R* B, int64_t N, int64_t levels, const ResidentShape& s,
+                                  const ResidentSync& y, const Coefs<R>& c, cudaStream_t st);
+
+}  // namespace swp
