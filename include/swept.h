@@ -90,16 +90,18 @@ typedef struct {
 /* How swp_advance_ex runs the swept scheme. */
 typedef enum {
     SWP_LAUNCH_AUTO = 0,        /* library choice, from measurement.  With the
-                                   default width and block size, heat and KS
-                                   run in one launch that keeps the grid on
-                                   chip (halo tiles in registers, exchanged
-                                   between co-resident blocks) where that is
-                                   the faster form: in FP64 up to 2^17 points,
-                                   beyond that heat up to about 10^6; in FP32
-                                   up to about 2*10^6, and in tiles of the same
+                                   default width and block size, an advance
+                                   runs in one launch that keeps the grid on
+                                   chip (halo tiles in registers or shared
+                                   memory, exchanged between co-resident
+                                   blocks) where that is the faster form: heat
+                                   and KS in FP64 up to 2^17 points, beyond that
+                                   heat up to about 10^6; Euler up to about
+                                   330000 cells; heat and KS in FP32 up to about
+                                   2*10^6 points, and in tiles of the same
                                    kind, a launch per some ten levels, above.
-                                   Otherwise (wider FP64 grids, Euler, a given
-                                   width, a stream under capture): periodic heat
+                                   Otherwise (wider FP64 grids, a given width,
+                                   a stream under capture): periodic heat
                                    and KS with N a multiple of 32, CLUSTER up to
                                    N = 2048 (FP64) or 4096 (FP32), then
                                    REGISTER up to 2^15 for FP64 heat, 2^14

@@ -414,7 +414,10 @@ bool run_swept_resident(swp_problem* p, int64_t steps, swp_status* st)
 {
     if (!p->shape_known) {
         p->shape_known = true;
-        if (!resident_plan(p->desc.eq, p->esize, p->N, p->sms, max_smem(p->device), &p->shape)) p->shape.K = 0;
+        const bool fits = p->desc.eq == SWP_EULER
+                              ? resident_euler_plan(p->N, p->sms, max_smem(p->device), &p->shape)
+                              : resident_plan(p->desc.eq, p->esize, p->N, p->sms, max_smem(p->device), &p->shape);
+        if (!fits) p->shape.K = 0;
     }
     if (p->shape.K == 0) return false;
     const int64_t levels = steps * p->sub;
@@ -440,7 +443,9 @@ bool run_swept_resident(swp_problem* p, int64_t steps, swp_status* st)
         return false;
     }
     if (cap != cudaStreamCaptureStatusNone) return false;
-    const size_t bytes = 2 * sizeof(uint64_t) * resident_words(p->desc.eq, p->esize, p->N, p->shape);
+    const size_t bytes = 2 * sizeof(uint64_t) * (p->desc.eq == SWP_EULER
+                                                     ? resident_euler_words(p->N, p->shape)
+                                                     : resident_words(p->desc.eq, p->esize, p->N, p->shape));
     cudaError_t e = cudaSuccess;
     if (!p->words) {
         // the words, and the status word behind them
@@ -470,8 +475,12 @@ bool run_swept_resident(swp_problem* p, int64_t steps, swp_status* st)
     y.wait_offset = withheld_offset(p);
     y.wait_limit_ns = p->wait_limit_ns;
     y.status = (int*)((char*)p->words + bytes);
-    e = launch_swept_resident<R>(p->desc.eq, p->desc.bc, (const R*)p->rows[p->cur], (R*)p->rows[1 - p->cur], p->N,
-                                 levels, p->shape, y, coefs_of<R>(p), p->stream);
+    if (p->desc.eq == SWP_EULER)
+        e = launch_swept_resident_euler(p->desc.bc, (const double*)p->rows[p->cur], (double*)p->rows[1 - p->cur], p->N,
+                                        levels, p->shape, y, coefs_of<double>(p), p->stream);
+    else
+        e = launch_swept_resident<R>(p->desc.eq, p->desc.bc, (const R*)p->rows[p->cur], (R*)p->rows[1 - p->cur],
+                                     p->N, levels, p->shape, y, coefs_of<R>(p), p->stream);
     if (e == cudaErrorCooperativeLaunchTooLarge) {   // the device cannot hold all blocks at once
         cudaGetLastError();
         p->shape.K = 0;

@@ -51,68 +51,12 @@
 #include <algorithm>
 
 #include "geometry.cuh"
+#include "resident.cuh"
 #include "resident.h"
 
 namespace swp {
 
 namespace {
-
-// Hard cap on polls of one wait, in case the global timer does not advance.
-constexpr uint32_t kMaxPolls = 1u << 26;
-
-__device__ __forceinline__ uint64_t global_ns()
-{
-    uint64_t t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-    return t;
-}
-
-// Published words: data and sequence number in one 8-byte access (FP64: two
-// of them, each half of the value).
-template <typename R> struct Word;
-template <> struct Word<float> {
-    static constexpr int N64 = 1;
-    static __device__ __forceinline__ void put(uint64_t* p, float v, uint32_t seq)
-    {
-        const uint64_t w = (uint64_t)seq << 32 | __float_as_uint(v);
-        asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
-    }
-    static __device__ __forceinline__ bool get(const uint64_t* p, float& v, uint32_t seq)
-    {
-        uint64_t w;
-        asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
-        v = __uint_as_float((uint32_t)w);
-        return (uint32_t)(w >> 32) == seq;
-    }
-};
-template <> struct Word<double> {
-    static constexpr int N64 = 2;
-    static __device__ __forceinline__ void put(uint64_t* p, double v, uint32_t seq)
-    {
-        const uint64_t b = (uint64_t)__double_as_longlong(v), s = (uint64_t)seq << 32;
-        asm volatile("st.relaxed.gpu.global.v2.u64 [%0], {%1, %2};" ::"l"(p), "l"(s | (b & 0xffffffffu)),
-                     "l"(s | (b >> 32))
-                     : "memory");
-    }
-    static __device__ __forceinline__ bool get(const uint64_t* p, double& v, uint32_t seq)
-    {
-        uint64_t a, b;
-        asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
-        v = __longlong_as_double((long long)((b << 32) | (a & 0xffffffffu)));
-        return (uint32_t)(a >> 32) == seq && (uint32_t)(b >> 32) == seq;
-    }
-};
-
-// Point of [0, N) that stands for point g of the extended line.
-__device__ __forceinline__ int64_t fold(int64_t g, int64_t N, int bc)
-{
-    const int64_t per = bc == PERIODIC ? N : 2 * (N - 1);
-    if (g < 0 || g >= per) {
-        g %= per;
-        if (g < 0) g += per;
-    }
-    return g < N ? g : per - g;
-}
 
 // FP32 runs of a multiple of 4 points move as 16-byte vectors.
 template <typename R, int P>
@@ -249,12 +193,8 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 1 : 0) swept_resident_ke
         buf0[slot_at<R, P>(s)] = s < own + 2 * h ? A[fold(b0 - h + s, N, g.bc)] : R(0);
     if (g.exchanges > 0) {
         for (int e = tid; e < 2 * h; e += T) {
-            // 32-bit arithmetic: N K < 2^31 (resident_plan)
-            const int p = (int)fold(b0 - h + (e < h ? e : own + e), N, g.bc), n = (int)N;
-            const int o = ((p + 1) * K - 1) / n;   // the block that owns point p
-            const int ob = o * n / K;
-            const int on = (o + 1) * n / K - ob, at = p - ob;
-            hoff[e] = o * cap + (on <= 2 * pub || at < pub ? at : at - (on - 2 * pub));
+            const int p = (int)fold(b0 - h + (e < h ? e : own + e), N, g.bc);
+            hoff[e] = word_of(p, (int)N, K, pub, cap);
         }
     }
     __syncthreads();
@@ -275,35 +215,24 @@ __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 1 : 0) swept_resident_ke
             left -= n;
         }
         if (x >= g.exchanges) break;
-        const uint32_t seq = g.seq + (uint32_t)x + g.wait_offset;
-        uint64_t* words = g.words + (x & 1) * g.parity_words;
+        const uint32_t seq = g.sync.seq + (uint32_t)x + g.sync.wait_offset;
+        uint64_t* words = g.sync.words + (x & 1) * g.parity_words;
         {
             const int words_here = min(own, 2 * pub);
             for (int i = tid; i < words_here; i += T) {
                 const int o = i < pub || own <= 2 * pub ? i : own - 2 * pub + i;
                 Word<R>::put(words + (int64_t)(k * cap + i) * Word<R>::N64, cur[slot_at<R, P>(h + o)],
-                             g.seq + (uint32_t)x);
+                             g.sync.seq + (uint32_t)x);
             }
         }
         int fail = 0;
         for (int e = tid; e < 2 * h; e += T) {
             const uint64_t* w = words + (int64_t)hoff[e] * Word<R>::N64;
             R v;
-            uint32_t polls = 0;
-            uint64_t t0 = 0;
-            while (!Word<R>::get(w, v, seq)) {
-                if ((++polls & 255u) == 0) {
-                    const uint64_t now = global_ns();
-                    if (t0 == 0) t0 = now;
-                    if (*reinterpret_cast<volatile int*>(g.status) != 0 || now - t0 > g.wait_limit_ns ||
-                        polls > kMaxPolls) {
-                        atomicExch(g.status, 1);
-                        fail = 1;
-                        break;
-                    }
-                }
+            if (!wait_word<R>(w, seq, g.sync, v)) {
+                fail = 1;
+                break;
             }
-            if (fail) break;
             cur[slot_at<R, P>(e < h ? e : own + e)] = v;
         }
         if (__syncthreads_or(fail)) return;
@@ -508,12 +437,8 @@ cudaError_t launch_swept_resident(int eq, int bc, const R* A, R* B, int64_t N, i
     g.exchanges = resident_exchanges(s, levels);
     g.last = (int)(levels - g.exchanges * g.E);
     g.bc = bc;
-    g.words = y.words;
+    g.sync = y;
     g.parity_words = y.words ? (int64_t)resident_words(eq, (int)sizeof(R), N, s) : 0;
-    g.seq = y.seq;
-    g.wait_offset = y.wait_offset;
-    g.wait_limit_ns = y.wait_limit_ns;
-    g.status = y.status;
     const size_t smem = smem_of((int)sizeof(R), s.P, g.slots, g.h);
     g.buf_elems = buffer_elems((int)sizeof(R), s.P, g.slots);
     const void* fn = kernel_of<R>(eq, s.P);

@@ -1,5 +1,6 @@
-// The resident form of a single heat / KS advance (resident.cu): launch
-// interface between the C-ABI layer (api.cu) and the kernel.  Internal header.
+// The resident form of a single advance (resident.cu, Euler: resident_euler.cu):
+// launch interface between the C-ABI layer (api.cu) and the kernels.  Internal
+// header.
 #pragma once
 
 #include <cstdint>
@@ -34,10 +35,7 @@ struct ResidentGeom {
     int pub, cap;          // points published at each end of a block, words per block
     int bc, last;          // boundary; levels after the last exchange
     int64_t exchanges, parity_words;
-    uint64_t* words;
-    uint32_t seq, wait_offset;
-    uint64_t wait_limit_ns;
-    int* status;
+    ResidentSync sync;
 };
 // The shape with the least estimated time per level, false when N does not fit.
 bool resident_plan(int eq, int esize, int64_t N, int sms, size_t max_smem, ResidentShape* out);
@@ -48,5 +46,13 @@ int64_t resident_exchanges(const ResidentShape& s, int64_t levels);
 template <typename R>
 cudaError_t launch_swept_resident(int eq, int bc, const R* A, R* B, int64_t N, int64_t levels, const ResidentShape& s,
                                   const ResidentSync& y, const Coefs<R>& c, cudaStream_t st);
+
+// The same for Euler (FP64): cells in shared memory, P and warps unused, L
+// levels per exchange, M = 1.
+bool resident_euler_plan(int64_t N, int sms, size_t max_smem, ResidentShape* out);
+size_t resident_euler_words(int64_t N, const ResidentShape& s);
+cudaError_t launch_swept_resident_euler(int bc, const double* A, double* B, int64_t N, int64_t levels,
+                                        const ResidentShape& s, const ResidentSync& y, const Coefs<double>& c,
+                                        cudaStream_t st);
 
 }  // namespace swp

@@ -1,0 +1,211 @@
+// Resident form of a single Euler advance: one launch, the cells in shared memory
+// from the first step to the last (resident.cu has the idea and the exchange).
+//
+// Each block owns a contiguous part of the grid and holds it with h = 2 L halo
+// cells on each side.  Level j of the L between two exchanges computes the
+// cells [2 j, W - 2 j) of the tile's W = own + 4 L, in the three passes of the
+// swept tiles: pressure and cached values per cell, one flux per interface,
+// the update.  After L levels the owned cells are current and the halos are
+// fetched again.  An update costs some hundred FP64 operations, so a level of
+// even one cell per lane outlasts an exchange many times over and L is
+// small; only the smallest grids, whose tiles do not fill the block's warps,
+// take more levels per exchange.
+//
+// What bounds it: the FP64 pipe.  A pass runs its rows of 32 cells on the SM's
+// four sub-partitions in turn, so its time goes with ceil(rows / 4); a grid of
+// 152 SMs x 128 cells or fewer has one row each, where the swept form took
+// 2H - 1 dependent levels per H levels of progress.  Clocks (2.07 GHz) per level
+// against the dataflow launch, Sod / limited everywhere: N = 4096 10700 / 10700
+// (21200 / 22600), 65536 23500 / 35700 (28000 / 48700), 200000 58300 / 102800
+// (62200 / 115100).  Grids whose cells do not fit shared memory (N above about
+// 330000) keep that launch.
+//
+// Dirichlet ends: the tile's slots beyond an end hold that end's ghost state in
+// both rows and are never updated (Appendix C's two ghost cells, and more of
+// the same).  Periodic ends wrap.
+#include <algorithm>
+
+#include "geometry.cuh"
+#include "resident.cuh"
+#include "resident.h"
+
+namespace swp {
+
+namespace {
+
+constexpr int kThreads = 256;
+
+__global__ void __launch_bounds__(kThreads) swept_resident_euler_kernel(const double* A, double* B, ResidentGeom g,
+                                                                        Coefs<double> cp)
+{
+    using R = double;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const Coefs<R> c = lane_coefs<R, EULER>(cp);
+    const Units<R> ku = make_units<R, EULER>();
+    const int T = kThreads, tid = threadIdx.x;
+    const int k = blockIdx.x, K = g.K, h = g.h, cap = g.cap, pub = g.pub;
+    const int64_t N = g.N;
+    const int64_t b0 = k * N / K;
+    const int own = (int)((k + 1) * N / K - b0), W = own + 2 * h, GW = W + 1;
+    R* row0 = reinterpret_cast<R*>(smem_raw);   // [3][W], even levels
+    R* row1 = row0 + 3 * W;                     // [3][W], odd levels
+    R* P = row1 + 3 * W;                        // pressures
+    R* Cc = P + W;                              // [3][W], cached (u, e, sqrt(rho))
+    R* G = Cc + 3 * W;                          // [3][W + 1]: interface between slots s - 1 and s
+    int* hoff = reinterpret_cast<int*>(G + 3 * GW);   // published word of each halo cell, -1: a ghost
+    // slots of the domain: all of them, or those between Dirichlet ends
+    int c_lo = 0, c_hi = W;
+    if (g.bc == DIRICHLET) {
+        if (b0 < h) c_lo = h - (int)b0;
+        if (N - (b0 - h) < W) c_hi = (int)(N - (b0 - h));
+    }
+    for (int s = tid; s < W; s += T) {
+        const bool left = s < c_lo, ghost = left || s >= c_hi;
+        const int64_t p = ghost ? 0 : fold(b0 - h + s, N, PERIODIC);
+#pragma unroll
+        for (int v = 0; v < 3; ++v) {
+            const R x = ghost ? (left ? c.ghost_l[v] : c.ghost_r[v]) : A[v * N + p];
+            row0[v * W + s] = x;
+            row1[v * W + s] = x;
+        }
+    }
+    if (g.exchanges > 0) {
+        for (int e = tid; e < 2 * h; e += T) {
+            const int s = e < h ? e : own + e;
+            hoff[e] = s < c_lo || s >= c_hi
+                          ? -1
+                          : word_of((int)fold(b0 - h + s, N, PERIODIC), (int)N, K, pub, cap);
+        }
+    }
+    __syncthreads();
+    for (int64_t x = 0;; ++x) {
+        const int levels = x < g.exchanges ? g.E : g.last;
+        for (int j = 1; j <= levels; ++j) {
+            const bool odd = j & 1;
+            const R* src = odd ? row0 : row1;
+            R* dst = odd ? row1 : row0;
+            const R kh = odd ? c.kh[0] : c.kh[1];
+            const int lo = 2 * j, hi = W - 2 * j;
+            for (int s = lo - 2 + tid; s < hi + 2; s += T)
+                P[s] = euler_cell(src[s], src[W + s], src[2 * W + s], c.gm1, Cc[s], Cc[W + s], Cc[2 * W + s], ku);
+            __syncthreads();
+            for (int s = lo + tid; s <= hi; s += T) {
+                const R qa[3] = {src[s - 1], src[W + s - 1], src[2 * W + s - 1]};
+                const R qb[3] = {src[s], src[W + s], src[2 * W + s]};
+                const R ca[3] = {Cc[s - 1], Cc[W + s - 1], Cc[2 * W + s - 1]};
+                const R cb[3] = {Cc[s], Cc[W + s], Cc[2 * W + s]};
+                R g3[3];
+                euler_interface_cached(qa, qb, P[s - 2], P[s - 1], P[s], P[s + 1], ca, cb, c.gm1, c.ggm1, g3, ku);
+                G[s] = g3[0];
+                G[GW + s] = g3[1];
+                G[2 * GW + s] = g3[2];
+            }
+            __syncthreads();
+            const int end = min(hi, c_hi);
+            for (int s = max(lo, c_lo) + tid; s < end; s += T) {
+#pragma unroll
+                for (int v = 0; v < 3; ++v)
+                    dst[v * W + s] =
+                        euler_update(G[v * GW + s + 1], G[v * GW + s], row0[v * W + s], kh, ku);   // base u^m
+            }
+            __syncthreads();
+        }
+        if (x >= g.exchanges) break;
+        const uint32_t seq = g.sync.seq + (uint32_t)x;
+        uint64_t* words = g.sync.words + (x & 1) * g.parity_words;
+        const int words_here = 3 * min(own, 2 * pub);
+        for (int i = tid; i < words_here; i += T) {
+            const int cell = i / 3, v = i - 3 * cell;
+            const int o = cell < pub || own <= 2 * pub ? cell : own - 2 * pub + cell;
+            Word<R>::put(words + 2 * ((int64_t)k * cap * 3 + i), row0[v * W + h + o], seq);
+        }
+        int fail = 0;
+        for (int i = tid; i < 6 * h; i += T) {
+            const int e = i / 3, v = i - 3 * e;
+            if (hoff[e] < 0) continue;
+            R q;
+            if (!wait_word<R>(words + 2 * ((int64_t)hoff[e] * 3 + v), seq + g.sync.wait_offset, g.sync, q)) {
+                fail = 1;
+                break;
+            }
+            row0[v * W + (e < h ? e : own + e)] = q;
+        }
+        if (__syncthreads_or(fail)) return;
+    }
+    for (int o = tid; o < own; o += T) {
+#pragma unroll
+        for (int v = 0; v < 3; ++v) B[v * N + b0 + o] = row0[v * W + h + o];
+    }
+}
+
+size_t smem_of(int own, int L)
+{
+    const size_t W = (size_t)own + 4 * (size_t)L;
+    return sizeof(double) * (6 * W + W + 3 * W + 3 * (W + 1)) + sizeof(int) * 4 * (size_t)L;
+}
+
+// Rows of 32 of n cells, in turns of the SM's four sub-partitions.
+int turns(int n) { return ((n + 31) / 32 + 3) / 4; }
+
+}  // namespace
+
+bool resident_euler_plan(int64_t N, int sms, size_t max_smem, ResidentShape* out)
+{
+    *out = ResidentShape();
+    if (N < 32 || sms < 1) return false;
+    const int K = (int)std::min<int64_t>(sms, std::max<int64_t>(1, N / 8));
+    if ((N + 1) * (K + 1) >= (int64_t)1 << 31) return false;
+    const int own = (int)((N + K - 1) / K);
+    double best = 0.0;
+    for (int L = 2; L <= 48; L += 2) {
+        const int W = own + 4 * L;
+        if (smem_of(own, L) > max_smem) break;
+        // FP64 operations of the passes (limited on some interfaces), their
+        // barriers, and an exchange
+        double clocks = 1700.0 + 20.0 * L;
+        for (int j = 1; j <= L; ++j)
+            clocks += 66.0 * (26 * turns(W - 4 * j + 4) + 80 * turns(W - 4 * j + 1) + 6 * turns(W - 4 * j)) + 300.0;
+        clocks /= L;
+        if (best == 0.0 || clocks < best) {
+            best = clocks;
+            out->K = K;
+            out->L = L;
+            out->M = 1;
+        }
+    }
+    return best > 0.0;
+}
+
+size_t resident_euler_words(int64_t N, const ResidentShape& s)
+{
+    const int own = (int)((N + s.K - 1) / s.K);
+    return (size_t)s.K * std::min(own, 2 * 2 * s.L) * 3 * 2;
+}
+
+cudaError_t launch_swept_resident_euler(int bc, const double* A, double* B, int64_t N, int64_t levels,
+                                        const ResidentShape& s, const ResidentSync& y, const Coefs<double>& c,
+                                        cudaStream_t st)
+{
+    ResidentGeom g{};
+    g.N = N;
+    g.K = s.K;
+    g.L = g.E = s.L;
+    g.h = 2 * s.L;
+    const int own = (int)((N + s.K - 1) / s.K);
+    g.pub = g.h;
+    g.cap = std::min(own, 2 * g.pub);
+    g.exchanges = resident_exchanges(s, levels);
+    g.last = (int)(levels - g.exchanges * g.E);
+    g.bc = bc;
+    g.sync = y;
+    g.parity_words = (int64_t)resident_euler_words(N, s);
+    const size_t smem = smem_of(own, s.L);
+    cudaError_t e = cudaFuncSetAttribute((const void*)swept_resident_euler_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    void* args[] = {(void*)&A, (void*)&B, (void*)&g, (void*)&c};
+    return cudaLaunchCooperativeKernel((const void*)swept_resident_euler_kernel, dim3((unsigned)s.K), dim3(kThreads),
+                                       args, smem, st);
+}
+
+}  // namespace swp

@@ -57,7 +57,25 @@ def test_default_launch_any_size(eq, bc, dtype, N):
             assert np.array_equal(p.read(), ref), steps
 
 
+@pytest.mark.parametrize("bc", ["dirichlet", "periodic"])
+@pytest.mark.parametrize("N", [32, 33, 61, 150, 1021, 4099, 16400, 20001])
+def test_default_launch_euler_any_size(bc, N):
+    """Tiles with ghost cells on one or both sides, halos over several blocks and
+    more than one period, one and several rows of cells per sub-partition."""
+    spec = spec_for("euler", bc, N)
+    u0 = state_for(spec, seed=N)
+    ref = u0.copy()
+    with S.Problem(spec, u0) as p:
+        for steps in (1, 5, 120 if N < 5000 else 40):
+            k0 = p.kernel_launches()
+            p.advance(steps, "swept")
+            assert p.kernel_launches() - k0 == 1
+            O.classic(oprob(spec), ref, steps)
+            assert np.array_equal(p.read(), ref), steps
+
+
 @pytest.mark.parametrize("eq,bc,N,dtype,steps", [
+    ("euler", "periodic", 200003, "f64", 30), ("euler", "dirichlet", 300001, "f64", 30),
     ("heat", "reflective", (1 << 17) + 1, "f64", 90), ("heat", "periodic", 400009, "f64", 60),
     ("heat", "periodic", (1 << 20) + 7, "f64", 70), ("heat", "reflective", 700001, "f32", 333),
     ("ks", "periodic", 300007, "f32", 120), ("ks", "periodic", 2097152, "f32", 100),
