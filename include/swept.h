@@ -230,9 +230,16 @@ size_t swp_memory_in_use(void);
  *   classic problem : a phase is one sub-timestep (Section 5.1), an item one
  *                     chunk of the balanced partition of [0, N) into
  *                     ceil(N / m) chunks of at most m points.
+ * Swept heat and KS problems given whole (not to the server's open rounds), with
+ * the default block size and no classic problem beside them, run in the on-chip
+ * form instead: a block keeps a tile of a problem for its whole advance, the
+ * problem's tiles exchanging halos (one cooperative launch; the node widths are
+ * checked and otherwise unused).  A problem with more tiles than the launch has
+ * blocks (about 900,000 points) sends the group to the table form.
  * Each problem's result is bit-identical to swp_advance with the same scheme
  * (and, swept, the same node width).  The table costs 12 bytes of device
- * memory per (problem, phase) task; this workspace is not counted against
+ * memory per (problem, phase) task, the on-chip form's halo words at most about
+ * 2 KB per 1000 points; this workspace is not counted against
  * swp_set_memory_budget.  A batch, like its problems, is used by one host
  * thread at a time.  The paper has no batched form. */
 typedef struct swp_batch swp_batch;

@@ -1013,12 +1013,12 @@ swp_status grow(void** p, size_t* cap, size_t bytes)
     return SWP_OK;
 }
 
-swp_status grow_tables(BatchTables& t, size_t inst_bytes, size_t ntasks, size_t nflags)
+swp_status grow_tables(BatchTables& t, size_t inst_bytes, size_t ntasks, size_t nctr, size_t nflags)
 {
     swp_status st;
     if ((st = grow(&t.insts, &t.insts_cap, inst_bytes)) != SWP_OK) return st;
     if ((st = grow((void**)&t.tasks, &t.tasks_cap, sizeof(int2) * ntasks)) != SWP_OK) return st;
-    if ((st = grow((void**)&t.ctr, &t.ctr_cap, sizeof(int) * (ntasks + 1))) != SWP_OK) return st;
+    if ((st = grow((void**)&t.ctr, &t.ctr_cap, sizeof(int) * nctr)) != SWP_OK) return st;
     return grow((void**)&t.flags, &t.flags_cap, sizeof(uint32_t) * nflags);
 }
 
@@ -1056,6 +1056,200 @@ swp_status check_chunk(const swp_problem* p, int m)
 // Estimated FP64-pipe operations per point of one level (sub-timestep).
 double level_cost(int eq) { return eq == SWP_HEAT ? 3.0 : (eq == SWP_KS ? 7.0 : 100.0); }
 
+// What a cached batch graph stands for: the form of its launch and, per problem,
+// its id (not the address: a new problem may reuse a destroyed one's), its
+// current row and its plan.
+std::vector<int64_t> batch_key(const std::vector<BatchItem>& items, int form, int threads)
+{
+    std::vector<int64_t> key;
+    key.reserve(items.size() * 7 + 2);
+    key.push_back(form);
+    key.push_back(threads);
+    for (const auto& it : items) {
+        key.push_back((int64_t)it.p->id);
+        key.push_back(it.p->cur);
+        key.push_back(it.kind);
+        key.push_back(it.s.n);
+        key.push_back(it.s.T);
+        key.push_back(it.p_lo);
+        key.push_back(it.p_hi);
+    }
+    return key;
+}
+
+// Replay the graph of this key, if there is one.
+bool batch_replay(swp_batch* b, const std::vector<int64_t>& key, swp_status* st)
+{
+    for (auto& g : b->graphs)
+        if (g.key == key) {
+            const cudaError_t e = cudaGraphLaunch(g.exec, b->stream);
+            *st = e == cudaSuccess ? SWP_OK : cuda_fail(e, "batch graph launch");
+            if (e != cudaSuccess) return true;
+            b->launches++;
+            for (auto* p : g.all) p->launches++;
+            for (auto* p : g.flip) p->cur = 1 - p->cur;
+            return true;
+        }
+    return false;
+}
+
+// Upload a launch's tables and run it: zero nctr counters and nflags flag words,
+// then launch(tables, stream), on the batch's stream or captured as a graph
+// with tables of its own under `key`.
+template <typename Launch>
+swp_status batch_launch(swp_batch* b, const std::vector<BatchItem>& items, std::vector<int64_t> key, const void* insts,
+                        size_t inst_bytes, const std::vector<int2>& tasks, size_t nctr, size_t nflags, bool graph,
+                        Launch launch)
+{
+    BatchGraph gnew;
+    BatchTables& t = graph ? gnew.t : b->t;
+    const size_t task_bytes = sizeof(int2) * tasks.size();
+    swp_status st = grow_tables(t, inst_bytes, tasks.size(), nctr, nflags);
+    if (st != SWP_OK) {
+        if (graph) gnew.t.release();
+        return st;
+    }
+    // upload through the pinned staging buffer once its previous upload is done
+    cudaError_t e = cudaEventSynchronize(b->staged);
+    if (e == cudaSuccess && b->stage_cap < inst_bytes + task_bytes) {
+        if (b->stage) cudaFreeHost(b->stage);
+        b->stage = nullptr;
+        b->stage_cap = 0;
+        const size_t want = inst_bytes + task_bytes + (inst_bytes + task_bytes) / 2 + 256;
+        e = cudaMallocHost(&b->stage, want);
+        if (e == cudaSuccess) b->stage_cap = want;
+    }
+    if (e == cudaSuccess) {
+        unsigned char* stg = (unsigned char*)b->stage;
+        std::memcpy(stg, insts, inst_bytes);
+        std::memcpy(stg + inst_bytes, tasks.data(), task_bytes);
+        e = cudaMemcpyAsync(t.insts, stg, inst_bytes, cudaMemcpyHostToDevice, b->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(t.tasks, stg + inst_bytes, task_bytes, cudaMemcpyHostToDevice, b->stream);
+        if (e == cudaSuccess) e = cudaEventRecord(b->staged, b->stream);
+    }
+    if (e != cudaSuccess) {
+        if (graph) gnew.t.release();
+        return cuda_fail(e, "batch table upload");
+    }
+    auto run = [&](cudaStream_t s) {
+        cudaError_t r = cudaMemsetAsync(t.ctr, 0, sizeof(int) * nctr, s);
+        if (r == cudaSuccess && nflags > 0) r = cudaMemsetAsync(t.flags, 0, sizeof(uint32_t) * nflags, s);
+        return r == cudaSuccess ? launch(t, s) : r;
+    };
+    if (!graph) {
+        e = run(b->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "batch launch");
+    } else {
+        // the uploads above are ordinary stream work; the graph holds the rest
+        if (!b->capture_stream) {
+            e = cudaStreamCreateWithFlags(&b->capture_stream, cudaStreamNonBlocking);
+            if (e != cudaSuccess) {
+                gnew.t.release();
+                return cuda_fail(e, "capture stream");
+            }
+        }
+        cudaGraph_t cg = nullptr;
+        e = cudaStreamBeginCapture(b->capture_stream, cudaStreamCaptureModeRelaxed);
+        if (e == cudaSuccess) {
+            const cudaError_t e1 = run(b->capture_stream);
+            e = cudaStreamEndCapture(b->capture_stream, &cg);
+            if (e1 != cudaSuccess) e = e1;
+        }
+        if (e == cudaSuccess) e = cudaGraphInstantiate(&gnew.exec, cg, 0);
+        if (cg) cudaGraphDestroy(cg);
+        if (e == cudaSuccess) e = cudaGraphLaunch(gnew.exec, b->stream);
+        if (e != cudaSuccess) {
+            if (gnew.exec) cudaGraphExecDestroy(gnew.exec);
+            cudaStreamSynchronize(b->stream);
+            gnew.t.release();
+            return cuda_fail(e, "batch graph capture");
+        }
+        gnew.key = std::move(key);
+        for (const auto& it : items) {
+            gnew.all.push_back(it.p);
+            if (it.flip) gnew.flip.push_back(it.p);
+        }
+        if (b->graphs.size() >= 8) {
+            // its last replay may still run: wait before freeing its tables
+            cudaStreamSynchronize(b->stream);
+            cudaGraphExecDestroy(b->graphs.front().exec);
+            b->graphs.front().t.release();
+            b->graphs.erase(b->graphs.begin());
+        }
+        b->graphs.push_back(std::move(gnew));
+    }
+    b->launches++;
+    for (const auto& it : items) {
+        it.p->launches++;
+        if (it.flip) it.p->cur = 1 - it.p->cur;
+    }
+    return SWP_OK;
+}
+
+// The batched resident launch of whole heat / KS advances (resident_batch.cu).
+// False (nothing done) when a problem has more tiles than the launch has blocks,
+// or the launch cannot run cooperatively: the dataflow launch takes them then.
+constexpr int kFormResident = 100;   // batch_key form, beside the dataflow modes
+
+template <typename R>
+bool resident_batch_group(swp_batch* b, const std::vector<BatchItem>& plans, bool graph, swp_status* st)
+{
+    const int own = resident_batch_own((int)sizeof(R));
+    const int resident = resident_batch_blocks<R>(b->sms);
+    int coop = 0;
+    if (resident <= 0 || cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, b->device) != cudaSuccess || !coop)
+        return false;
+    int64_t ntiles = 0, words = 0;
+    for (const auto& it : plans) {
+        const int64_t K = (it.p->N + own - 1) / own;
+        if (it.kind != BATCH_SWEPT || K > resident || it.s.T >= ((int64_t)1 << 31)) return false;
+        ntiles += K;
+    }
+    if (ntiles >= (int64_t)1 << 30) return false;
+    std::vector<BatchItem> items = plans;
+    for (auto& it : items) it.flip = true;   // from one row to the other
+    std::vector<int64_t> key;
+    if (graph) {
+        key = batch_key(items, kFormResident, 0);
+        if (batch_replay(b, key, st)) return true;
+    }
+    std::vector<ResidentInst<R>> insts(items.size());
+    std::vector<std::pair<double, int>> order(items.size());   // longest advance first
+    for (size_t i = 0; i < items.size(); ++i) {
+        const swp_problem* p = items[i].p;
+        ResidentInst<R>& in = insts[i];
+        in.A = (const R*)p->rows[p->cur];
+        in.B = (R*)p->rows[1 - p->cur];
+        in.eq = p->desc.eq;
+        in.g = resident_batch_geom<R>(p->desc.eq, p->desc.bc, p->N, items[i].s.T);
+        in.word_off = words;
+        in.c = coefs_of<R>(p);
+        if (in.g.K > 1) words += 2 * in.g.parity_words;
+        order[i] = {-(double)items[i].s.T * level_cost(p->desc.eq), (int)i};
+    }
+    std::stable_sort(order.begin(), order.end());
+    std::vector<int2> tiles;
+    tiles.reserve((size_t)ntiles);
+    for (const auto& o : order) {
+        for (int k = 0; k < insts[o.second].g.K; ++k) tiles.push_back(make_int2(o.second, k));
+        insts[o.second].last_tile = (int)tiles.size() - 1;
+    }
+    ResidentBatchWork w;
+    w.ntiles = (int)ntiles;
+    w.status = b->status;
+    w.wait_limit_ns = b->wait_limit_ns;
+    const int blocks = (int)std::min<int64_t>(resident, ntiles);
+    *st = batch_launch(b, items, std::move(key), insts.data(), sizeof(ResidentInst<R>) * insts.size(), tiles, 1,
+                       2 * (size_t)words, graph, [&](const BatchTables& t, cudaStream_t s) {
+                           w.tiles = t.tasks;
+                           w.next_tile = t.ctr;
+                           w.words = (uint64_t*)t.flags;
+                           return launch_swept_resident_batch<R>((const ResidentInst<R>*)t.insts, w, blocks, s);
+                       });
+    return true;
+}
+
 // One persistent launch of the items (one equation group and dtype).  status,
 // wait_offset and wait_limit override the batch's status word and bounded-wait
 // settings (the single-problem persistent launch and its test hook).
@@ -1066,28 +1260,9 @@ swp_status batch_group(swp_batch* b, const std::vector<BatchItem>& items, int mo
 {
     std::vector<int64_t> key;
     if (graph) {
-        key.reserve(items.size() * 5 + 2);
-        key.push_back(mode);
-        key.push_back(threads);
-        for (const auto& it : items) {
-            // the id, not the address: a new problem may reuse a destroyed one's
-            key.push_back((int64_t)it.p->id);
-            key.push_back(it.p->cur);
-            key.push_back(it.kind);
-            key.push_back(it.s.n);
-            key.push_back(it.s.T);
-            key.push_back(it.p_lo);
-            key.push_back(it.p_hi);
-        }
-        for (auto& g : b->graphs)
-            if (g.key == key) {
-                cudaError_t e = cudaGraphLaunch(g.exec, b->stream);
-                if (e != cudaSuccess) return cuda_fail(e, "batch graph launch");
-                b->launches++;
-                for (auto* p : g.all) p->launches++;
-                for (auto* p : g.flip) p->cur = 1 - p->cur;
-                return SWP_OK;
-            }
+        key = batch_key(items, mode, threads);
+        swp_status st = SWP_OK;
+        if (batch_replay(b, key, &st)) return st;
     }
     std::vector<BatchInst<R>> insts(items.size());
     int64_t flags = 0, items_total = 0;
@@ -1144,47 +1319,12 @@ swp_status batch_group(swp_batch* b, const std::vector<BatchItem>& items, int mo
     });
     if (flags >= (int64_t)1 << 30) return fail(SWP_EINVAL, "batch too large for one launch");
     const size_t ntasks = keys.size();
-    const size_t inst_bytes = sizeof(BatchInst<R>) * insts.size();
-    const size_t task_bytes = sizeof(int2) * ntasks;
-
-    BatchGraph gnew;
-    BatchTables& t = graph ? gnew.t : b->t;
-    swp_status st = grow_tables(t, inst_bytes, ntasks, (size_t)flags);
-    if (st != SWP_OK) {
-        if (graph) gnew.t.release();
-        return st;
-    }
-    // upload through the pinned staging buffer once its previous upload is done
-    cudaError_t e = cudaEventSynchronize(b->staged);
-    if (e == cudaSuccess && b->stage_cap < inst_bytes + task_bytes) {
-        if (b->stage) cudaFreeHost(b->stage);
-        b->stage = nullptr;
-        b->stage_cap = 0;
-        const size_t want = inst_bytes + task_bytes + (inst_bytes + task_bytes) / 2 + 256;
-        e = cudaMallocHost(&b->stage, want);
-        if (e == cudaSuccess) b->stage_cap = want;
-    }
-    if (e == cudaSuccess) {
-        unsigned char* stg = (unsigned char*)b->stage;
-        std::memcpy(stg, insts.data(), inst_bytes);
-        int2* tk = (int2*)(stg + inst_bytes);
-        for (size_t i = 0; i < ntasks; ++i) tk[i] = make_int2(keys[i].inst, keys[i].phase);
-        e = cudaMemcpyAsync(t.insts, stg, inst_bytes, cudaMemcpyHostToDevice, b->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(t.tasks, tk, task_bytes, cudaMemcpyHostToDevice, b->stream);
-        if (e == cudaSuccess) e = cudaEventRecord(b->staged, b->stream);
-    }
-    if (e != cudaSuccess) {
-        if (graph) gnew.t.release();
-        return cuda_fail(e, "batch table upload");
-    }
+    std::vector<int2> tasks(ntasks);
+    for (size_t i = 0; i < ntasks; ++i) tasks[i] = make_int2(keys[i].inst, keys[i].phase);
     BatchWork w;
-    w.tasks = t.tasks;
-    w.cur_task = t.ctr;
-    w.task_ctr = t.ctr + 1;
-    w.status = status ? status : b->status;
     w.ntasks = (int)ntasks;
     w.smem_bytes = smem;
-    w.flags = t.flags;
+    w.status = status ? status : b->status;
     w.wait_limit_ns = wait_limit ? wait_limit : b->wait_limit_ns;
     w.wait_offset = wait_offset;
     bool reg = false, cls = false;
@@ -1194,66 +1334,19 @@ swp_status batch_group(swp_batch* b, const std::vector<BatchItem>& items, int mo
     }
     int bps = swept_batch_blocks_per_sm<R>(mode, reg, cls, smem, threads);
     if (max_blocks_per_sm > 0 && bps > max_blocks_per_sm) bps = max_blocks_per_sm;
-    if (bps <= 0) {
-        if (graph) gnew.t.release();
+    if (bps <= 0)
         return fail(SWP_EINVAL, "batch kernel does not fit (%zu bytes of shared memory, threads=%d)", smem, threads);
-    }
     int64_t blocks = (int64_t)b->sms * bps;
     if (blocks > items_total) blocks = items_total;
-    const BatchInst<R>* dinsts = (const BatchInst<R>*)t.insts;
-    if (!graph) {
-        e = cudaMemsetAsync(t.ctr, 0, sizeof(int) * (ntasks + 1), b->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(t.flags, 0, sizeof(uint32_t) * (size_t)flags, b->stream);
-        if (e == cudaSuccess) e = launch_swept_batch<R>(mode, reg, cls, dinsts, w, threads, (int)blocks, b->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "batch launch");
-    } else {
-        // the uploads above are ordinary stream work; the graph holds the rest
-        if (!b->capture_stream) {
-            e = cudaStreamCreateWithFlags(&b->capture_stream, cudaStreamNonBlocking);
-            if (e != cudaSuccess) {
-                gnew.t.release();
-                return cuda_fail(e, "capture stream");
-            }
-        }
-        cudaGraph_t cg = nullptr;
-        e = cudaStreamBeginCapture(b->capture_stream, cudaStreamCaptureModeRelaxed);
-        if (e == cudaSuccess) {
-            cudaError_t e1 = cudaMemsetAsync(t.ctr, 0, sizeof(int) * (ntasks + 1), b->capture_stream);
-            if (e1 == cudaSuccess)
-                e1 = cudaMemsetAsync(t.flags, 0, sizeof(uint32_t) * (size_t)flags, b->capture_stream);
-            if (e1 == cudaSuccess) e1 = launch_swept_batch<R>(mode, reg, cls, dinsts, w, threads, (int)blocks, b->capture_stream);
-            e = cudaStreamEndCapture(b->capture_stream, &cg);
-            if (e1 != cudaSuccess) e = e1;
-        }
-        if (e == cudaSuccess) e = cudaGraphInstantiate(&gnew.exec, cg, 0);
-        if (cg) cudaGraphDestroy(cg);
-        if (e == cudaSuccess) e = cudaGraphLaunch(gnew.exec, b->stream);
-        if (e != cudaSuccess) {
-            if (gnew.exec) cudaGraphExecDestroy(gnew.exec);
-            cudaStreamSynchronize(b->stream);
-            gnew.t.release();
-            return cuda_fail(e, "batch graph capture");
-        }
-        gnew.key = std::move(key);
-        for (const auto& it : items) {
-            gnew.all.push_back(it.p);
-            if (it.flip) gnew.flip.push_back(it.p);
-        }
-        if (b->graphs.size() >= 8) {
-            // its last replay may still run: wait before freeing its tables
-            cudaStreamSynchronize(b->stream);
-            cudaGraphExecDestroy(b->graphs.front().exec);
-            b->graphs.front().t.release();
-            b->graphs.erase(b->graphs.begin());
-        }
-        b->graphs.push_back(std::move(gnew));
-    }
-    b->launches++;
-    for (const auto& it : items) {
-        it.p->launches++;
-        if (it.flip) it.p->cur = 1 - it.p->cur;
-    }
-    return SWP_OK;
+    return batch_launch(b, items, std::move(key), insts.data(), sizeof(BatchInst<R>) * insts.size(), tasks, ntasks + 1,
+                        (size_t)flags, graph, [&](const BatchTables& t, cudaStream_t s) {
+                            w.tasks = t.tasks;
+                            w.cur_task = t.ctr;
+                            w.task_ctr = t.ctr + 1;
+                            w.flags = t.flags;
+                            return launch_swept_batch<R>(mode, reg, cls, (const BatchInst<R>*)t.insts, w, threads,
+                                                         (int)blocks, s);
+                        });
 }
 
 swp_status persistent_via_batch(swp_problem* p, const SweptPlan& s, int threads)
@@ -1286,12 +1379,20 @@ swp_status persistent_via_batch(swp_problem* p, const SweptPlan& s, int threads)
 }
 
 // One group launch per (equation group, dtype) of the given items.
-swp_status launch_groups(swp_batch* b, std::vector<BatchItem> (&groups)[2][2], int threads, bool graph)
+// whole: the items are whole advances (not ranges of open ones).
+swp_status launch_groups(swp_batch* b, std::vector<BatchItem> (&groups)[2][2], int threads, bool graph, bool whole)
 {
     for (int g = 0; g < 2; ++g)
         for (int dt = 0; dt < 2; ++dt) {
             if (groups[g][dt].empty()) continue;
             const int mode = g == 1 ? SWP_EULER : SWP_HEAT;
+            swp_status rs = SWP_OK;
+            if (whole && g == 0 && threads == 0 &&
+                (dt == SWP_F64 ? resident_batch_group<double>(b, groups[g][dt], graph, &rs)
+                               : resident_batch_group<float>(b, groups[g][dt], graph, &rs))) {
+                if (rs != SWP_OK) return rs;
+                continue;
+            }
             // default block, measured on the batched heat+KS workload: 128
             // threads in FP64; one warp per node in FP32, where a level's
             // barrier is the cost that matters
@@ -1362,7 +1463,7 @@ swp_status batch_advance(swp_batch* b, swp_problem* const* problems, const int64
     }
     if (threads < 0 || threads > max_threads || threads % 32)
         return fail(SWP_EINVAL, "threads must be 0 or a multiple of 32 in [32, %d]", max_threads);
-    return launch_groups(b, groups, threads, launch == SWP_LAUNCH_GRAPH);
+    return launch_groups(b, groups, threads, launch == SWP_LAUNCH_GRAPH, true);
 }
 
 // Node width for N points from a target width w: N split into
@@ -1487,7 +1588,7 @@ swp_status batch_advance_phases(swp_batch* b, const PhaseRange* ranges, int coun
                   (classic ? (p->desc.eq == SWP_HEAT && (it.s.T & 1)) : (it.s.top & 1) != 0);
         groups[p->desc.eq == SWP_EULER ? 1 : 0][p->desc.dtype].push_back(it);
     }
-    return launch_groups(b, groups, threads, false);
+    return launch_groups(b, groups, threads, false, false);
 }
 
 swp_status set_error(swp_status s, const char* msg) { return fail(s, "%s", msg); }

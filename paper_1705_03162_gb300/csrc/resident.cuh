@@ -86,6 +86,10 @@ __device__ __forceinline__ bool wait_word(const uint64_t* w, uint32_t seq, const
     while (!Word<R>::get(w, v, seq)) {
         if ((++polls & 255u) == 0) {
             const uint64_t now = clock_ns();
+            if (y.claimed && *reinterpret_cast<const volatile int*>(y.claimed) <= y.last_tile) {
+                t0 = now;
+                polls = 0;
+            }
             if (t0 == 0) t0 = now;
             if (*reinterpret_cast<volatile int*>(y.status) != 0 || now - t0 > y.wait_limit_ns ||
                 polls > kMaxWordPolls) {

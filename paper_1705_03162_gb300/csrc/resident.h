@@ -27,6 +27,11 @@ struct ResidentSync {
     uint32_t wait_offset;  // 0; a test hook sets it so that no wait can succeed
     uint64_t wait_limit_ns;
     int* status;           // != 0: a wait gave up
+    // batched form: tiles claimed so far, and the problem's last tile in the list.
+    // Until it is claimed a wait is for another problem's tile to end (whose own
+    // waits are bounded), and its limit has not begun.
+    const int* claimed = nullptr;
+    int last_tile = 0;
 };
 struct ResidentGeom {
     int64_t N;
@@ -46,6 +51,32 @@ int64_t resident_exchanges(const ResidentShape& s, int64_t levels);
 template <typename R>
 cudaError_t launch_swept_resident(int eq, int bc, const R* A, R* B, int64_t N, int64_t levels, const ResidentShape& s,
                                   const ResidentSync& y, const Coefs<R>& c, cudaStream_t st);
+
+// Many heat and KS problems in one launch (resident_batch.cu): a block keeps a
+// tile, (problem, k), for its whole advance.
+template <typename R> struct ResidentInst {
+    const R* A;
+    R* B;
+    int eq;
+    int64_t word_off;      // of the problem's first published word
+    int last_tile;         // the problem's last tile in the list
+    ResidentGeom g;        // sync unset
+    Coefs<R> c;
+};
+struct ResidentBatchWork {
+    const int2* tiles;     // (problem, tile), a problem's tiles together
+    int ntiles;
+    int* next_tile;        // zeroed per launch
+    uint64_t* words;       // zeroed per launch
+    int* status;
+    uint64_t wait_limit_ns;
+};
+int resident_batch_own(int esize);   // the most points a tile owns
+template <typename R> ResidentGeom resident_batch_geom(int eq, int bc, int64_t N, int64_t levels);
+template <typename R> int resident_batch_blocks(int sms);   // blocks resident at once
+template <typename R>
+cudaError_t launch_swept_resident_batch(const ResidentInst<R>* insts, const ResidentBatchWork& w, int blocks,
+                                        cudaStream_t s);
 
 // The same for Euler (FP64): cells in shared memory, P and warps unused, L
 // levels per exchange, M = 1.

@@ -141,3 +141,31 @@ def test_withheld_words_time_out_and_recover():
         p.write(u0)
         p.advance(300, "swept")
         assert np.array_equal(p.read(), _oracle(spec, u0, 300))
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_batch_of_whole_advances(dtype):
+    """The batched resident launch: problems of one tile (their halos are their
+    own points, over several periods for the smallest), of two, and of many,
+    more tiles than the launch has blocks, advances of one level, of an odd
+    number, of one exchange exactly and of many; twice, the second time replayed
+    from a graph with the rows exchanged."""
+    torch = pytest.importorskip("torch")
+    stream = torch.cuda.Stream()
+    kinds = [("heat", "periodic"), ("heat", "reflective"), ("ks", "periodic")]
+    sizes = [16, 21, 100, 735, 745, 1489, 1857, 2049, 4099, 30011, 100003]
+    steps = [1, 3, 8, 64, 97, 130]
+    cases = [(eq, bc, N, steps[(i + j) % 6]) for i, N in enumerate(sizes) for j, (eq, bc) in enumerate(kinds)]
+    cases += [("heat", "periodic", 3000 + 17 * i, 20 + i) for i in range(400)]
+    specs = [spec_for(eq, bc, N) for eq, bc, N, _ in cases]
+    u0 = [state_for(s, _np(dtype), seed=i) for i, s in enumerate(specs)]
+    probs = [S.Problem(s, u, dtype, stream=stream) for s, u in zip(specs, u0)]
+    with S.Batch(stream) as b:
+        for _ in range(3):
+            b.advance_ex(probs, [c[3] for c in cases], ["swept"] * len(cases), launch="graph")
+        b.advance(probs, [c[3] for c in cases])
+        b.synchronize()
+        assert b.kernel_launches() == 4
+    for (eq, bc, N, st), s, u, p in zip(cases, specs, u0, probs):
+        assert np.array_equal(p.read(), _oracle(s, u, 4 * st)), (eq, bc, N, st)
+        p.close()
