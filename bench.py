@@ -89,14 +89,14 @@ def alu_roofline(updates: float, seconds: float, eq: str, dtype: str) -> dict:
 NCU_TRAFFIC = {
     # dram__bytes_read.sum + dram__bytes_write.sum of the whole 10^4-step solve in
     # one dataflow launch: a one-pass capture of the benchmark's own timed launch
-    "swept_batch_kernel<double,KS> n=1024 threads=256": {"src": "36cee9459e5c736b", "bytes_per_launch": 11540000},
+    "swept_batch_kernel<double,KS> n=1024 threads=256": {"src": "560c5446004eac6c", "bytes_per_launch": 11830000},
 }
 # Issue-slot use of the batched FP32 launch from one ncu capture (the 4096
-# instances of the batched workload, every node width 2048 fitted to N): warp
+# instances of the batched workload; the on-chip tiles of resident_batch.cu): warp
 # instructions issued over 4 per SM per cycle, keyed like the traffic record
 # and reported when the timed batch runs that width.
-NCU_ISSUE_FP32_BATCH = {"src": "36cee9459e5c736b", "width": 2048, "issue_frac": 0.699, "issue_active": 0.701,
-                        "fma_pipe": 0.401}
+NCU_ISSUE_FP32_BATCH = {"src": "560c5446004eac6c", "width": 2048, "issue_frac": 0.712, "issue_active": 0.713,
+                        "fma_pipe": 0.634}
 KERNEL_OF_LAUNCH = {"per_phase": "swept_phase_kernel", "graph": "swept_phase_kernel",
                     "persistent": "swept_batch_kernel", "auto": "swept_batch_kernel"}
 
@@ -111,7 +111,8 @@ def _code_only(text: str) -> str:
 
 def _kernel_src_hash() -> str:
     h = hashlib.sha256()
-    for f in ("swept.cu", "geometry.cuh", "scheme.cuh", "launch.h"):
+    for f in ("swept.cu", "geometry.cuh", "scheme.cuh", "launch.h", "resident.h", "resident.cuh", "resident_tile.cuh",
+              "resident_batch.cu"):
         with open(os.path.join(ROOT, "paper_1705_03162_gb300", "csrc", f), encoding="utf-8") as fh:
             h.update(_code_only(fh.read()).encode())
     return h.hexdigest()[:16]

@@ -6,9 +6,8 @@
 // loading) in shared memory.  Both evaluate the shared point update of
 // scheme.cuh.
 // Euler evaluates each interface flux once per tile (P per cell, G per
-// interface) instead of twice per cell, and reuses each cell's velocity,
-// specific energy and sqrt(rho) on the interface sides the limiter leaves
-// first order.
+// interface) instead of twice per cell, runs the limiter once per cell, and
+// reuses the values of first-order cells on both their interfaces.
 #include "launch.h"
 
 namespace swp {
@@ -58,10 +57,12 @@ __global__ void __launch_bounds__(256) classic_kernel(const R* __restrict__ src,
         R* P = sm + NV * SW;        // pressure of every staged cell
         R* G = P + SW;              // G[v][l]: interface between tile cells l-1 and l
         const int GW = TILE + 1;
-        R* Cc = G + 3 * GW;         // cached (u, e, sqrt(rho)) of staged cell s at Cc[k SW + s]
-        for (int s = threadIdx.x; s < SW; s += T) {
-            P[s] = euler_cell(sm[s], sm[SW + s], sm[2 * SW + s], c.gm1, Cc[s], Cc[SW + s], Cc[2 * SW + s], ku);
-        }
+        R* Cc = G + 3 * GW;         // kept values (euler_limit) of staged cell s at Cc[k SW + s]
+        for (int s = threadIdx.x; s < SW; s += T)
+            P[s] = euler_cell(sm[s], sm[SW + s], sm[2 * SW + s], c.gm1, Cc[s], Cc[SW + s], ku);
+        __syncthreads();
+        for (int s = 1 + threadIdx.x; s < SW - 1; s += T)
+            euler_limit<false>(P[s - 1], P[s], P[s + 1], sm[s], Cc[s], Cc[SW + s], Cc[2 * SW + s], ku);
         __syncthreads();
         for (int l = threadIdx.x; l < GW; l += T) {
             if (t0 + l > N) break;
@@ -71,7 +72,7 @@ __global__ void __launch_bounds__(256) classic_kernel(const R* __restrict__ src,
             const R ca[3] = {Cc[sb - 1], Cc[SW + sb - 1], Cc[2 * SW + sb - 1]};
             const R cb[3] = {Cc[sb], Cc[SW + sb], Cc[2 * SW + sb]};
             R g3[3];
-            euler_interface_cached(qa, qb, P[sb - 2], P[sb - 1], P[sb], P[sb + 1], ca, cb, c.gm1, c.ggm1, g3, ku);
+            euler_interface(qa, qb, P[sb - 1], P[sb], ca, cb, c.gm1, c.ggm1, g3, ku);
             G[l] = g3[0];
             G[GW + l] = g3[1];
             G[2 * GW + l] = g3[2];

@@ -3,8 +3,8 @@
 //
 // Each block owns a contiguous part of the grid and holds it with h = 2 L halo
 // cells on each side.  Level j of the L between two exchanges computes the
-// cells [2 j, W - 2 j) of the tile's W = own + 4 L, in the three passes of the
-// swept tiles: pressure and cached values per cell, one flux per interface,
+// cells [2 j, W - 2 j) of the tile's W = own + 4 L, in the four passes of the
+// swept tiles: pressure per cell, the limiter per cell, one flux per interface,
 // the update.  After L levels the owned cells are current and the halos are
 // fetched again.  An update costs some hundred FP64 operations, so a level of
 // even one cell per lane outlasts an exchange many times over and L is
@@ -15,9 +15,9 @@
 // four sub-partitions in turn, so its time goes with ceil(rows / 4); a grid of
 // 152 SMs x 128 cells or fewer has one row each, where the swept form took
 // 2H - 1 dependent levels per H levels of progress.  Clocks (2.07 GHz) per level
-// against the dataflow launch, Sod / limited everywhere: N = 4096 10700 / 10700
-// (21200 / 22600), 65536 23500 / 35700 (28000 / 48700), 200000 58300 / 102800
-// (62200 / 115100).  Grids whose cells do not fit shared memory (N above about
+// against the dataflow launch, Sod / limited everywhere: N = 4096 8100 / 8200
+// (21200 / 22600 when this form came), 65536 22600 / 32900 (28000 / 48700), 200000
+// 56200 / 94700 (62200 / 115100).  Grids whose cells do not fit shared memory (N above about
 // 330000) keep that launch.
 //
 // Dirichlet ends: the tile's slots beyond an end hold that end's ghost state in
@@ -35,6 +35,11 @@ namespace {
 
 constexpr int kThreads = 256;
 
+// SPLIT: for tiles of at most two rows of cells, whose passes would leave
+// sub-partitions idle: a cell's pressure and its sqrt(rho), and the two sides of
+// an interface, are tasks of their own on different warps (N = 4096: 8100 against
+// 10330 clocks per level).
+template <bool SPLIT>
 __global__ void __launch_bounds__(kThreads) swept_resident_euler_kernel(const double* A, double* B, ResidentGeom g,
                                                                         Coefs<double> cp)
 {
@@ -50,9 +55,10 @@ __global__ void __launch_bounds__(kThreads) swept_resident_euler_kernel(const do
     R* row0 = reinterpret_cast<R*>(smem_raw);   // [3][W], even levels
     R* row1 = row0 + 3 * W;                     // [3][W], odd levels
     R* P = row1 + 3 * W;                        // pressures
-    R* Cc = P + W;                              // [3][W], cached (u, e, sqrt(rho))
+    R* Cc = P + W;                              // [3][W], kept values (euler_limit)
     R* G = Cc + 3 * W;                          // [3][W + 1]: interface between slots s - 1 and s
-    int* hoff = reinterpret_cast<int*>(G + 3 * GW);   // published word of each halo cell, -1: a ghost
+    R* S = G + 3 * GW;                          // SPLIT: [2][8][W + 1], the sides of every interface
+    int* hoff = reinterpret_cast<int*>(S + (SPLIT ? 16 * GW : 0));   // published word of each halo cell, -1: a ghost
     // slots of the domain: all of them, or those between Dirichlet ends
     int c_lo = 0, c_hi = W;
     if (g.bc == DIRICHLET) {
@@ -86,16 +92,62 @@ __global__ void __launch_bounds__(kThreads) swept_resident_euler_kernel(const do
             R* dst = odd ? row1 : row0;
             const R kh = odd ? c.kh[0] : c.kh[1];
             const int lo = 2 * j, hi = W - 2 * j;
-            for (int s = lo - 2 + tid; s < hi + 2; s += T)
-                P[s] = euler_cell(src[s], src[W + s], src[2 * W + s], c.gm1, Cc[s], Cc[W + s], Cc[2 * W + s], ku);
+            if constexpr (SPLIT) {
+                // whole warps for each, so that none runs both
+                const int n = (hi - lo + 4 + 31) & ~31;
+                for (int t = tid; t < 2 * n; t += T) {
+                    const int s = lo - 2 + (t < n ? t : t - n);
+                    if (s >= hi + 2) continue;
+                    if (t < n) P[s] = euler_cell(src[s], src[W + s], src[2 * W + s], c.gm1, Cc[s], Cc[W + s], ku);
+                    else Cc[2 * W + s] = Fp<R>::sqrt(src[s]);
+                }
+            } else {
+                for (int s = lo - 2 + tid; s < hi + 2; s += T)
+                    P[s] = euler_cell(src[s], src[W + s], src[2 * W + s], c.gm1, Cc[s], Cc[W + s], ku);
+            }
             __syncthreads();
-            for (int s = lo + tid; s <= hi; s += T) {
+            for (int s = lo - 1 + tid; s < hi + 1; s += T)
+                euler_limit<SPLIT>(P[s - 1], P[s], P[s + 1], src[s], Cc[s], Cc[W + s], Cc[2 * W + s], ku);
+            __syncthreads();
+            if constexpr (SPLIT) {
+                const int n = hi - lo + 1;
+                for (int t = tid; t < 2 * n; t += T) {
+                    const int right = t >= n, s = lo + (right ? t - n : t);
+                    const int a = s - 1 + right, b = s - right;   // the side's cell, and the other
+                    const R qc[3] = {src[a], src[W + a], src[2 * W + a]};
+                    const R qo[3] = {src[b], src[W + b], src[2 * W + b]};
+                    const R cc[3] = {Cc[a], Cc[W + a], Cc[2 * W + a]};
+                    R q[3], f1, f2, u, e, w;
+                    euler_side(qc, qo, P[a], cc, right ? cc[1] : cc[0], c.gm1, q, f1, f2, u, e, w, ku);
+                    R* o = S + right * 8 * GW + s;
+                    o[0] = q[0];
+                    o[GW] = q[1];
+                    o[2 * GW] = q[2];
+                    o[3 * GW] = f1;
+                    o[4 * GW] = f2;
+                    o[5 * GW] = right ? Fp<R>::mul(w, u, ku) : u;
+                    o[6 * GW] = right ? Fp<R>::mul(w, e, ku) : e;
+                    o[7 * GW] = w;
+                }
+                __syncthreads();
+                for (int s = lo + tid; s <= hi; s += T) {
+                    const R* l = S + s;
+                    const R* r = l + 8 * GW;
+                    const R ql[3] = {l[0], l[GW], l[2 * GW]}, qr[3] = {r[0], r[GW], r[2 * GW]};
+                    R g3[3];
+                    euler_join(ql, l[3 * GW], l[4 * GW], l[5 * GW], l[6 * GW], l[7 * GW], qr, r[3 * GW], r[4 * GW],
+                               r[5 * GW], r[6 * GW], r[7 * GW], c.ggm1, g3, ku);
+                    G[s] = g3[0];
+                    G[GW + s] = g3[1];
+                    G[2 * GW + s] = g3[2];
+                }
+            } else for (int s = lo + tid; s <= hi; s += T) {
                 const R qa[3] = {src[s - 1], src[W + s - 1], src[2 * W + s - 1]};
                 const R qb[3] = {src[s], src[W + s], src[2 * W + s]};
                 const R ca[3] = {Cc[s - 1], Cc[W + s - 1], Cc[2 * W + s - 1]};
                 const R cb[3] = {Cc[s], Cc[W + s], Cc[2 * W + s]};
                 R g3[3];
-                euler_interface_cached(qa, qb, P[s - 2], P[s - 1], P[s], P[s + 1], ca, cb, c.gm1, c.ggm1, g3, ku);
+                euler_interface(qa, qb, P[s - 1], P[s], ca, cb, c.gm1, c.ggm1, g3, ku);
                 G[s] = g3[0];
                 G[GW + s] = g3[1];
                 G[2 * GW + s] = g3[2];
@@ -138,10 +190,10 @@ __global__ void __launch_bounds__(kThreads) swept_resident_euler_kernel(const do
     }
 }
 
-size_t smem_of(int own, int L)
+size_t smem_of(int own, int L, bool split)
 {
     const size_t W = (size_t)own + 4 * (size_t)L;
-    return sizeof(double) * (6 * W + W + 3 * W + 3 * (W + 1)) + sizeof(int) * 4 * (size_t)L;
+    return sizeof(double) * (6 * W + W + 3 * W + (split ? 19 : 3) * (W + 1)) + sizeof(int) * 4 * (size_t)L;
 }
 
 // Rows of 32 of n cells, in turns of the SM's four sub-partitions.
@@ -157,22 +209,28 @@ bool resident_euler_plan(int64_t N, int sms, size_t max_smem, ResidentShape* out
     if ((N + 1) * (K + 1) >= (int64_t)1 << 31) return false;
     const int own = (int)((N + K - 1) / K);
     double best = 0.0;
-    for (int L = 2; L <= 48; L += 2) {
-        const int W = own + 4 * L;
-        if (smem_of(own, L) > max_smem) break;
-        // FP64 operations of the passes (limited on some interfaces), their
-        // barriers, and an exchange
-        double clocks = 1700.0 + 20.0 * L;
-        for (int j = 1; j <= L; ++j)
-            clocks += 66.0 * (26 * turns(W - 4 * j + 4) + 80 * turns(W - 4 * j + 1) + 6 * turns(W - 4 * j)) + 300.0;
-        clocks /= L;
-        if (best == 0.0 || clocks < best) {
-            best = clocks;
-            out->K = K;
-            out->L = L;
-            out->M = 1;
+    for (int split = 0; split < 2; ++split)
+        for (int L = 2; L <= 48; L += 2) {
+            const int W = own + 4 * L;
+            if (smem_of(own, L, split) > max_smem) break;
+            // FP64 operations of the passes (limited on some interfaces), their
+            // barriers and latencies, and an exchange
+            double clocks = 1700.0 + 20.0 * L;
+            for (int j = 1; j <= L; ++j) {
+                const int n = W - 4 * j;
+                const int flux = split ? 28 * turns(2 * n + 2) + 33 * turns(n + 1) : 82 * turns(n + 1);
+                const int cell = split ? 10 * turns(2 * ((n + 4 + 31) & ~31)) + 12 * turns(n + 2) : 11 * turns(n + 4) + 20 * turns(n + 2);
+                clocks += 66.0 * (cell + flux + 6 * turns(n)) + (split ? 700.0 : 500.0);
+            }
+            clocks /= L;
+            if (best == 0.0 || clocks < best) {
+                best = clocks;
+                out->K = K;
+                out->L = L;
+                out->M = 1;
+                out->P = split;
+            }
         }
-    }
     return best > 0.0;
 }
 
@@ -199,13 +257,12 @@ cudaError_t launch_swept_resident_euler(int bc, const double* A, double* B, int6
     g.bc = bc;
     g.sync = y;
     g.parity_words = (int64_t)resident_euler_words(N, s);
-    const size_t smem = smem_of(own, s.L);
-    cudaError_t e = cudaFuncSetAttribute((const void*)swept_resident_euler_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = smem_of(own, s.L, s.P != 0);
+    const void* fn = s.P ? (const void*)swept_resident_euler_kernel<true> : (const void*)swept_resident_euler_kernel<false>;
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&A, (void*)&B, (void*)&g, (void*)&c};
-    return cudaLaunchCooperativeKernel((const void*)swept_resident_euler_kernel, dim3((unsigned)s.K), dim3(kThreads),
-                                       args, smem, st);
+    return cudaLaunchCooperativeKernel(fn, dim3((unsigned)s.K), dim3(kThreads), args, smem, st);
 }
 
 }  // namespace swp

@@ -194,118 +194,113 @@ __device__ __forceinline__ bool same_sign(R a, R b)
     return (ua << 1) != 0 && (ub << 1) != 0 && ((ua ^ ub) >> top) == 0;
 }
 
-// min(num/den, 1) for num, den nonzero with the same sign.  When
-// |num| >= |den| the quotient rounds to >= 1, so the division is skipped.
-template <typename R>
-__device__ __forceinline__ R limited_ratio(R num, R den)
-{
-    const auto mag = ~(decltype(fbits(num)))0 >> 1;
-    return (fbits(num) & mag) >= (fbits(den) & mag) ? R(1) : Fp<R>::div(num, den);
-}
+// What a level keeps per cell beside its pressure.  The limiter (Eqs. Pratio,
+// limitleft, limitright) compares the pressure differences on the two sides of
+// a cell, and both states that the cell gives, QL = Q + min(ratio, 1)/2 (Q+ - Q) on
+// its right and QR = Q + min(1/ratio, 1)/2 (Q- - Q) on its left, ratio =
+// (p+ - p)/(p - p-), are limited or first order together: the ratio lies in
+// (0, inf) exactly when both differences are nonzero with the same sign.
+//  - first order (uniform regions, extrema): both states are the cell's own, so
+//    its velocity, specific energy e = E/rho and sqrt(rho) serve both interfaces;
+//  - limited: min(ratio, 1)/2 and min(1/ratio, 1)/2, of which one is 1/2 (a
+//    quotient of |num| >= |den| rounds to at least 1), so one division serves both;
+//    the third value is kLimited, which no sqrt yields.
+// Against evaluating each interface side on its own this drops a division, and
+// on limited cells the cell's own square root: 200000 cells limited everywhere,
+// 100 steps, 9.93 to 8.34 ms.
+constexpr uint64_t kLimitedBits = 0xbff0000000000000ull;   // -1.0
 
-// Limited states at the interface between cells a (left) and b (right)
-// (Eqs. Pratio, limitleft, limitright): the ratio at cell a is
-// (pb - pa)/(pa - pam) and gives QL = Qa + min(ratio, 1)/2 (Qb - Qa) when it
-// lies in (0, inf); the inverse ratio at cell b, (pb - pa)/(pbp - pb), gives
-// QR = Qb + min(inverse, 1)/2 (Qa - Qb); otherwise first order.
-// lfirst / rfirst: the side was left first order (a copy of its cell).
-template <typename R>
-__device__ __forceinline__ void euler_reconstruct(const R qa[3], const R qb[3], R pam, R pa,
-                                                  R pb, R pbp, R ql[3], R qr[3], bool& lfirst, bool& rfirst,
-                                                  const Units<R>& k)
-{
-    using F = Fp<R>;
-    R num = F::sub(pb, pa, k), den = F::sub(pa, pam, k);
-    lfirst = !same_sign(num, den);
-    if (!lfirst) {
-        R h = F::mul(F::half(k), limited_ratio(num, den), k);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) ql[c] = F::fma(h, F::sub(qb[c], qa[c], k), qa[c]);
-    } else {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) ql[c] = qa[c];
-    }
-    R num2 = F::sub(pbp, pb, k);
-    rfirst = !same_sign(num2, num);
-    if (!rfirst) {
-        R h = F::mul(F::half(k), limited_ratio(num, num2), k);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) qr[c] = F::fma(h, F::sub(qa[c], qb[c], k), qb[c]);
-    } else {
-#pragma unroll
-        for (int c = 0; c < 3; ++c) qr[c] = qb[c];
-    }
-}
+__device__ __forceinline__ bool euler_limited(double third) { return (uint64_t)__double_as_longlong(third) == kLimitedBits; }
+__device__ __forceinline__ bool euler_limited(float third) { return third == -1.0f; }
 
-// G = 2 Flux from the limited states: F(QR) + F(QL) + r_sp (QL - QR), with
-// F(Q) = (rho u, rho u^2 + P, u (E + P)) (Eq. EulerF) and spectral radius
-// r_sp = sqrt(gamma (gamma-1) (e_sp - u_sp^2/2)) + |u_sp| from sqrt(rho)-weighted
-// Roe averages of u and of e = E/rho (gamma P_sp / rho_sp with
-// P_sp = (gamma-1) rho_sp (e_sp - u_sp^2/2)).  Divisions by rho and by the
-// weight sum are multiplications by correctly rounded reciprocals.
-//
-// Per-cell values are reused.  Where the limiter leaves a side first order
-// (uniform regions: the pressure difference is 0), the side state is its
-// cell's state, and the flux's pressure, velocity, specific energy e = E/rho
-// and sqrt(rho) of that side are the cell's own.  euler_cell forms them once
-// per cell with exactly the operations a limited side's state gets, so
-// reusing them gives the same bits.
+// First pass: pressure, and the velocity and specific energy of a cell.
 template <typename R>
-__device__ __forceinline__ R euler_cell(R r, R m, R E, R gm1, R& u, R& e, R& s, const Units<R>& k)
+__device__ __forceinline__ R euler_cell(R r, R m, R E, R gm1, R& u, R& e, const Units<R>& k)
 {
     R ir;
     const R p = euler_pressure(r, m, E, gm1, u, ir, k);
     e = Fp<R>::mul(E, ir, k);
-    s = Fp<R>::sqrt(r);
     return p;
 }
 
-// Pressure, velocity, e and sqrt(rho) of a limited side state q.
-template <typename R>
-__device__ __forceinline__ R euler_side(const R q[3], R gm1, R& u, R& e, R& s, const Units<R>& k)
-{
-    return euler_cell(q[0], q[1], q[2], gm1, u, e, s, k);
-}
-
-// ca / cb: (u, e, sqrt(rho)) of cells a and b (as euler_cell forms them).
-template <typename R>
-__device__ __forceinline__ void euler_interface_cached(const R qa[3], const R qb[3], R pam, R pa, R pb,
-                                                       R pbp, const R ca[3], const R cb[3], R gm1, R ggm1,
-                                                       R G[3], const Units<R>& k)
+// Second pass, with the pressures of the cell and its neighbours: c0, c1 hold
+// (u, e) from the first pass and become, with c2, the cell's kept values.
+// ROOT: c2 holds sqrt(r) already.
+template <bool ROOT, typename R>
+__device__ __forceinline__ void euler_limit(R pm, R p, R pp, R r, R& c0, R& c1, R& c2, const Units<R>& k)
 {
     using F = Fp<R>;
-    R ql[3], qr[3];
-    bool lfirst, rfirst;
-    euler_reconstruct(qa, qb, pam, pa, pb, pbp, ql, qr, lfirst, rfirst, k);
-    R pl, ul, el, sl, pr, ur, er, sr;
-    if (lfirst) {
-        pl = pa;
-        ul = ca[0];
-        el = ca[1];
-        sl = ca[2];
-    } else {
-        pl = euler_side(ql, gm1, ul, el, sl, k);
+    const R dp = F::sub(pp, p, k), dm = F::sub(p, pm, k);
+    if (same_sign(dp, dm)) {
+        const auto mag = ~(decltype(fbits(dp)))0 >> 1;
+        const auto ap = fbits(dp) & mag, am = fbits(dm) & mag;
+        const bool steep = ap >= am;   // ratio >= 1
+        const R h = ap == am ? R(0.5) : F::mul(F::half(k), F::div(steep ? dm : dp, steep ? dp : dm), k);
+        c0 = steep ? R(0.5) : h;
+        c1 = steep ? h : R(0.5);
+        c2 = R(-1);
+    } else if (!ROOT) {
+        c2 = F::sqrt(r);
     }
-    if (rfirst) {
-        pr = pb;
-        ur = cb[0];
-        er = cb[1];
-        sr = cb[2];
+}
+
+// One side of an interface: its state q (the cell's, or limited towards the
+// other cell's state qo with factor h), velocity, e and sqrt(rho), and the flux
+// F(q) = (rho u, f1, f2) = (rho u, rho u^2 + P, u (E + P)) (Eq. EulerF).
+template <typename R>
+__device__ __forceinline__ void euler_side(const R qc[3], const R qo[3], R pc, const R c[3], R h, R gm1, R q[3], R& f1,
+                                           R& f2, R& u, R& e, R& s, const Units<R>& k)
+{
+    using F = Fp<R>;
+    R p;
+    if (euler_limited(c[2])) {
+#pragma unroll
+        for (int v = 0; v < 3; ++v) q[v] = F::fma(h, F::sub(qo[v], qc[v], k), qc[v]);
+        p = euler_cell(q[0], q[1], q[2], gm1, u, e, k);
+        s = F::sqrt(q[0]);
     } else {
-        pr = euler_side(qr, gm1, ur, er, sr, k);
+#pragma unroll
+        for (int v = 0; v < 3; ++v) q[v] = qc[v];
+        p = pc;
+        u = c[0];
+        e = c[1];
+        s = c[2];
     }
-    R fl1 = F::fma(ql[1], ul, pl);
-    R fl2 = F::mul(ul, F::add(ql[2], pl, k), k);
-    R fr1 = F::fma(qr[1], ur, pr);
-    R fr2 = F::mul(ur, F::add(qr[2], pr, k), k);
+    f1 = F::fma(q[1], u, p);
+    f2 = F::mul(u, F::add(q[2], p, k), k);
+}
+
+// G = 2 Flux from the two sides, F(QR) + F(QL) + r_sp (QL - QR), with spectral
+// radius r_sp = sqrt(gamma (gamma-1) (e_sp - u_sp^2/2)) + |u_sp| from
+// sqrt(rho)-weighted Roe averages of u and of e = E/rho (gamma P_sp / rho_sp with
+// P_sp = (gamma-1) rho_sp (e_sp - u_sp^2/2)).  Divisions by rho and by the
+// weight sum are multiplications by correctly rounded reciprocals.
+// su, se: sr ur and sr er.
+template <typename R>
+__device__ __forceinline__ void euler_join(const R ql[3], R fl1, R fl2, R ul, R el, R sl, const R qr[3], R fr1, R fr2,
+                                           R su, R se, R sr, R ggm1, R G[3], const Units<R>& k)
+{
+    using F = Fp<R>;
     R iw = F::rcp(F::add(sl, sr, k));
-    R usp = F::mul(F::fma(sl, ul, F::mul(sr, ur, k)), iw, k);
-    R esp = F::mul(F::fma(sl, el, F::mul(sr, er, k)), iw, k);
+    R usp = F::mul(F::fma(sl, ul, su), iw, k);
+    R esp = F::mul(F::fma(sl, el, se), iw, k);
     R c2 = F::mul(ggm1, F::fma(F::mul(F::mhalf(k), usp, k), usp, esp), k);
     R rsp = F::add(F::sqrt(c2), F::abs(usp), k);
     G[0] = F::fma(rsp, F::sub(ql[0], qr[0], k), F::add(qr[1], ql[1], k));
     G[1] = F::fma(rsp, F::sub(ql[1], qr[1], k), F::add(fr1, fl1, k));
     G[2] = F::fma(rsp, F::sub(ql[2], qr[2], k), F::add(fr2, fl2, k));
+}
+
+// Third pass, the interface between cells a (left) and b (right) with kept values
+// ca and cb.
+template <typename R>
+__device__ __forceinline__ void euler_interface(const R qa[3], const R qb[3], R pa, R pb, const R ca[3], const R cb[3],
+                                                R gm1, R ggm1, R G[3], const Units<R>& k)
+{
+    R ql[3], qr[3], fl1, fl2, ul, el, sl, fr1, fr2, ur, er, sr;
+    euler_side(qa, qb, pa, ca, ca[0], gm1, ql, fl1, fl2, ul, el, sl, k);
+    euler_side(qb, qa, pb, cb, cb[1], gm1, qr, fr1, fr2, ur, er, sr, k);
+    euler_join(ql, fl1, fl2, ul, el, sl, qr, fr1, fr2, Fp<R>::mul(sr, ur, k), Fp<R>::mul(sr, er, k), sr, ggm1, G, k);
 }
 
 // Finite-volume RK2 stage: out = base - (h/dx)(Flux_{i+1/2} - Flux_{i-1/2})
