@@ -39,15 +39,14 @@
 // What bounds it.  FP64: its pipe, at 66 clocks per warp-wide FMA; with one warp
 // per SM sub-partition the chain of a level (KS N = 1024: 550 of 670 clocks),
 // and the exchange of about 1450 clocks between blocks.  FP32: instruction
-// issue; 94 % of the instructions are the point updates' own (KS, 2000003
-// points; 67 % of issue slots used, the rest lost to register-bank limits of
-// three-operand FMAs).  Measured per advance against the forms that were the
+// issue; 94 % of the instructions are the point updates' own, and the slots that
+// eligible warps leave unused are lost to their register operands (Pair).  Measured per advance against the forms that were the
 // default before (cluster, Register and Shared graphs, per-phase FP32):
 //   heat FP64 N = 1024, 4096 steps      1196 -> 610 us
 //   heat FP64 reflective 50001, 2000    1559 -> 807 us
 //   KS FP64 10007, 2000 steps           3224 -> 1575 us
 //   heat FP32 2^17, 4000 steps          1080 -> 178 us
-//   KS FP32 2000003, 1000 steps         3710 -> 1158 us
+//   KS FP32 2000003, 1000 steps         3710 -> 1014 us
 #include <algorithm>
 
 #include "resident.h"
@@ -59,12 +58,10 @@ namespace {
 
 template <typename R, int EQ, int P>
 __global__ void __launch_bounds__(512, sizeof(R) == 4 ? 1 : 0)
-    swept_resident_kernel(const R* A, R* B, ResidentGeom g, Coefs<R> cp)
+    swept_resident_kernel(const R* A, R* B, ResidentGeom g, Coefs<R> c)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const Coefs<R> c = lane_coefs<R, EQ>(cp);
-    const Units<R> ku = make_units<R, EQ>();
-    resident_tile<R, EQ, P, false>(A, B, g, (int)blockIdx.x, smem_raw, c, ku);
+    resident_tile<R, EQ, P, EQ == KS && kVector<R, P>, false>(A, B, g, (int)blockIdx.x, smem_raw, c);
 }
 
 // Kernel of (precision, equation, points per thread), or NULL.
@@ -130,7 +127,7 @@ namespace {
 // shared memory every L levels (170 to 1000) and the exchange between blocks
 // every L M levels (1450 and the polls of its halo).  FP64 is its pipe's time
 // (66 clocks per warp-wide FMA) and a latency that a second warp per SM
-// sub-partition hides; FP32 is issue, at 1.1 (heat) and 1.36 (KS) slots per
+// sub-partition hides; FP32 is issue, at 1.1 (heat) and about 1.36 (KS) slots per
 // operation, above the latency of a level's shuffles and chain.
 double level_clocks(int eq, int esize, int warps, int P, int L, int M, int h)
 {

@@ -31,7 +31,8 @@ namespace {
 // heat and KS problems of 2^10..2^16 points.  Smaller blocks lose less at their
 // barriers when they share an SM (FP64, P = 12: 58.1 ms with 2 warps, 61.2 with 4,
 // 59.0 with 1, whose tiles have more halo); FP32 rounds stale whole lanes of
-// 16-point vectors (P = 16: 11.1 ms; 8: 12.4, 12: 12.0, 24: 12.0).
+// 16-point vectors (P = 16: 11.1 ms; 8: 12.4, 12: 11.6, 20: 11.2, 28: 11.4; KS runs
+// in pairs, which gain in the single launch, 12.2).
 template <typename R> struct Tile;
 template <> struct Tile<float> {
     static constexpr int P = 16, EDGE = 16, M = 3, THREADS = 128, BLOCKS_PER_SM = 4;
@@ -63,12 +64,8 @@ __global__ void __launch_bounds__(Tile<R>::THREADS, Tile<R>::BLOCKS_PER_SM)
         g.sync.claimed = w.next_tile;
         g.sync.last_tile = in.last_tile;
         bool ok;
-        if (in.eq == HEAT)
-            ok = resident_tile<R, HEAT, P, true>(in.A, in.B, g, tk.y, smem_raw, lane_coefs<R, HEAT>(in.c),
-                                                 make_units<R, HEAT>());
-        else
-            ok = resident_tile<R, KS, P, true>(in.A, in.B, g, tk.y, smem_raw, lane_coefs<R, KS>(in.c),
-                                               make_units<R, KS>());
+        if (in.eq == HEAT) ok = resident_tile<R, HEAT, P, false, true>(in.A, in.B, g, tk.y, smem_raw, in.c);
+        else ok = resident_tile<R, KS, P, false, true>(in.A, in.B, g, tk.y, smem_raw, in.c);
         if (!ok) break;
         __syncthreads();   // tile_s and the buffers are free again
     }
