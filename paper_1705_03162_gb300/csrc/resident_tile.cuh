@@ -235,8 +235,8 @@ __device__ __forceinline__ Units<V> run_units()
 
 // The whole advance of tile k of g.K: points [k N / K, (k + 1) N / K) from row A to
 // row B.  False when a wait gave up (all threads together).
-// SELF: g.K may be 1, whose halos are its own points.
-template <typename R, int EQ, int P, bool PAIRS, bool SELF>
+// BATCH: g.K may be 1, whose halos are its own points.
+template <typename R, int EQ, int P, bool PAIRS, bool BATCH>
 __device__ __forceinline__ bool resident_tile(const R* A, R* B, const ResidentGeom& g, int k, unsigned char* smem_raw,
                                               const Coefs<R>& launch_coefs)
 {
@@ -255,9 +255,10 @@ __device__ __forceinline__ bool resident_tile(const R* A, R* B, const ResidentGe
     const int edge = RAD * g.L;
     // the lane's run starts at this tile slot; slot s is point b0 - h + s
     const int w0 = (tid >> 5) * (32 * P - 2 * edge), s0 = w0 + lane * P;
-    const bool active = w0 + edge < own + 2 * h;   // the warp's valid points reach the tile's
-    const int cap = g.cap, pub = g.pub;            // published points per block: all, or pub at each end
-    const bool self = SELF && K == 1;
+    // a batch's tiles vary in length: warps whose valid points lie past the tile's rest
+    const bool active = !BATCH || w0 + edge < own + 2 * h;
+    const int cap = g.cap, pub = g.pub;   // published points per block: all, or pub at each end
+    const bool self = BATCH && K == 1;
     for (int s = tid; s < g.slots; s += T)
         cur[slot_at<R, P, PAIRS>(s)] = s < own + 2 * h ? A[fold(b0 - h + s, N, g.bc)] : R(0);
     if (g.exchanges > 0) {
