@@ -232,10 +232,13 @@ size_t swp_memory_in_use(void);
  *                     ceil(N / m) chunks of at most m points.
  * Swept heat and KS problems given whole (not to the server's open rounds), with
  * the default block size and no classic problem beside them, run in the on-chip
- * form instead: a block keeps a tile of a problem for its whole advance, the
- * problem's tiles exchanging halos (one cooperative launch; the node widths are
- * checked and otherwise unused).  A problem with more tiles than the launch has
- * blocks (about 900,000 points) sends the group to the table form.
+ * form where it is the faster one: a block keeps a tile of a problem for its
+ * whole advance, the problem's tiles exchanging halos (one cooperative launch).
+ * That is every FP32 group, and FP64 groups of few points (below about 80,000 in
+ * all) or many (above about 750,000); FP64 groups in between run the table form
+ * with its default widths.  In all these the given node widths are checked and
+ * otherwise unused.  A problem with more tiles than the launch has blocks (about
+ * 900,000 points) sends the group to the table form with the given widths.
  * Each problem's result is bit-identical to swp_advance with the same scheme
  * (and, swept, the same node width).  The table costs 12 bytes of device
  * memory per (problem, phase) task, the on-chip form's halo words at most about
@@ -251,7 +254,7 @@ swp_status swp_batch_create(void* cuda_stream, swp_batch** out);
 /* Advance problems[i] by n_steps[i] timesteps (swept), i < count.
  * points_per_block: per-problem node widths (any width swp_advance accepts),
  * or NULL / 0 entries for the tuned width of swp_autotune_width (else the
- * default rule; a problem too small for any node width runs as classic
+ * default rule, for Euler one that goes by the batch's cells; a problem too small for any node width runs as classic
  * items, with the same result).  threads: block
  * size (0 = 128 for FP64 and 32 for FP32; Euler at most 256).  Problems must be distinct.  Asynchronous;
  * SWP_ETIMEOUT surfaces at swp_batch_synchronize (wait bound as for

@@ -257,6 +257,22 @@ int width_for(const swp_problem* p, bool dataflow = false)
     return default_width(p, dataflow);
 }
 
+// Node width of an Euler problem among `cells` cells advancing together in a
+// dataflow launch: about 1500 nodes in all, 64 to 512 cells each.  Measured with
+// 128 threads, ms, for 64 / 128 / 256 / 512-cell nodes (256 threads) and for the
+// width of the problem alone: 8 problems of 6 k to 115 k cells 61 / 47 / 52 / 60, 66;
+// 40 of 1 k to 16 k 29.6 / 24.2 / 24.8 / 27.5, 30.7; one of 50 k 4.9 / 5.9 / 8.7 /
+// 10.8, 6.7; 3 of 130 k to 1 M 108 / 78 / 68 / 66, 65.
+int euler_batch_width(const swp_problem* p, int64_t cells)
+{
+    Tuned t;
+    if (tuned_of(p->desc, &t) && t.n_swept > 0 && check_width(p, t.n_swept) == SWP_OK) return t.n_swept;
+    const int64_t target = std::min(p->N / 2, std::max<int64_t>(64, std::min<int64_t>(512, cells / 1500)));
+    for (int n = (int)(target / 8 * 8); n >= 8; n -= 8)
+        if (check_width(p, n) == SWP_OK) return n;
+    return 0;
+}
+
 // Classic chunk width of a batched classic advance (points per item).
 int default_chunk(const swp_problem* p)
 {
@@ -1188,25 +1204,31 @@ swp_status batch_launch(swp_batch* b, const std::vector<BatchItem>& items, std::
 }
 
 // The batched resident launch of whole heat / KS advances (resident_batch.cu).
-// False (nothing done) when a problem has more tiles than the launch has blocks,
-// or the launch cannot run cooperatively: the dataflow launch takes them then.
+// False (nothing launched) when the dataflow launch takes them: a problem has more
+// tiles than the launch has blocks, the launch cannot run cooperatively, or the
+// dataflow launch is faster, for which the plans get their default widths.
 constexpr int kFormResident = 100;   // batch_key form, beside the dataflow modes
 
 template <typename R>
-bool resident_batch_group(swp_batch* b, const std::vector<BatchItem>& plans, bool graph, swp_status* st)
+bool resident_batch_group(swp_batch* b, std::vector<BatchItem>& plans, bool graph, swp_status* st)
 {
-    const int own = resident_batch_own((int)sizeof(R));
-    const int resident = resident_batch_blocks<R>(b->sms);
     int coop = 0;
-    if (resident <= 0 || cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, b->device) != cudaSuccess || !coop)
-        return false;
-    int64_t ntiles = 0, words = 0;
-    for (const auto& it : plans) {
-        const int64_t K = (it.p->N + own - 1) / own;
-        if (it.kind != BATCH_SWEPT || K > resident || it.s.T >= ((int64_t)1 << 31)) return false;
-        ntiles += K;
-    }
-    if (ntiles >= (int64_t)1 << 30) return false;
+    if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, b->device) != cudaSuccess || !coop) return false;
+    for (const auto& it : plans)
+        if (it.kind != BATCH_SWEPT || it.s.T >= ((int64_t)1 << 31)) return false;
+    std::vector<int64_t> points;
+    for (const auto& it : plans) points.push_back(it.p->N);
+    ResidentBatchShape shape;
+    const ResidentBatchFit fit = resident_batch_choose((int)sizeof(R), points, b->sms, &shape);
+    if (fit == RESIDENT_SLOWER)
+        for (auto& it : plans) {
+            const int n = width_for(it.p);
+            if (n == 0 || n == it.s.n) continue;
+            it.s = plan_swept(it.p, it.s.T / it.p->sub, n);
+            it.p_hi = it.s.n_phases;
+            it.flip = (it.s.top & 1) != 0;
+        }
+    if (fit != RESIDENT_FITS) return false;
     std::vector<BatchItem> items = plans;
     for (auto& it : items) it.flip = true;   // from one row to the other
     std::vector<int64_t> key;
@@ -1214,38 +1236,38 @@ bool resident_batch_group(swp_batch* b, const std::vector<BatchItem>& plans, boo
         key = batch_key(items, kFormResident, 0);
         if (batch_replay(b, key, st)) return true;
     }
-    std::vector<ResidentInst<R>> insts(items.size());
     std::vector<std::pair<double, int>> order(items.size());   // longest advance first
-    for (size_t i = 0; i < items.size(); ++i) {
+    for (size_t i = 0; i < items.size(); ++i)
+        order[i] = {-(double)items[i].s.T * level_cost(items[i].p->desc.eq), (int)i};
+    std::stable_sort(order.begin(), order.end());
+    std::vector<ResidentInst<R>> insts(items.size());
+    std::vector<int2> tiles;
+    int64_t words = 0;
+    for (const auto& o : order) {
+        const int i = o.second;
         const swp_problem* p = items[i].p;
         ResidentInst<R>& in = insts[i];
         in.A = (const R*)p->rows[p->cur];
         in.B = (R*)p->rows[1 - p->cur];
         in.eq = p->desc.eq;
-        in.g = resident_batch_geom<R>(p->desc.eq, p->desc.bc, p->N, items[i].s.T);
+        in.g = resident_batch_geom(p->desc.eq, (int)sizeof(R), p->desc.bc, p->N, items[i].s.T, shape);
         in.word_off = words;
         in.c = coefs_of<R>(p);
         if (in.g.K > 1) words += 2 * in.g.parity_words;
-        order[i] = {-(double)items[i].s.T * level_cost(p->desc.eq), (int)i};
-    }
-    std::stable_sort(order.begin(), order.end());
-    std::vector<int2> tiles;
-    tiles.reserve((size_t)ntiles);
-    for (const auto& o : order) {
-        for (int k = 0; k < insts[o.second].g.K; ++k) tiles.push_back(make_int2(o.second, k));
-        insts[o.second].last_tile = (int)tiles.size() - 1;
+        if ((int64_t)tiles.size() + in.g.K >= (int64_t)1 << 30) return false;
+        for (int k = 0; k < in.g.K; ++k) tiles.push_back(make_int2(i, k));
+        in.last_tile = (int)tiles.size() - 1;
     }
     ResidentBatchWork w;
-    w.ntiles = (int)ntiles;
+    w.ntiles = (int)tiles.size();
     w.status = b->status;
     w.wait_limit_ns = b->wait_limit_ns;
-    const int blocks = (int)std::min<int64_t>(resident, ntiles);
     *st = batch_launch(b, items, std::move(key), insts.data(), sizeof(ResidentInst<R>) * insts.size(), tiles, 1,
                        2 * (size_t)words, graph, [&](const BatchTables& t, cudaStream_t s) {
                            w.tiles = t.tasks;
                            w.next_tile = t.ctr;
                            w.words = (uint64_t*)t.flags;
-                           return launch_swept_resident_batch<R>((const ResidentInst<R>*)t.insts, w, blocks, s);
+                           return launch_swept_resident_batch<R>((const ResidentInst<R>*)t.insts, w, shape, s);
                        });
     return true;
 }
@@ -1418,6 +1440,9 @@ swp_status batch_advance(swp_batch* b, swp_problem* const* problems, const int64
         return fail(SWP_EINVAL, "current device differs from the batch's device");
     std::vector<BatchItem> groups[2][2];   // [heat+KS | Euler][dtype]
     int max_threads = 1024;
+    int64_t euler_cells = 0;
+    for (int32_t i = 0; i < count; ++i)
+        if (problems[i] && problems[i]->desc.eq == SWP_EULER && n_steps[i] > 0) euler_cells += problems[i]->N;
     for (int32_t i = 0; i < count; ++i) {
         swp_problem* p = problems[i];
         if (!p) return fail(SWP_EINVAL, "problem %d is NULL", i);
@@ -1439,7 +1464,7 @@ swp_status batch_advance(swp_batch* b, swp_problem* const* problems, const int64
         BatchItem it;
         it.p = p;
         if (scheme == SWP_SWEPT && n == 0) {
-            n = width_for(p);
+            n = p->desc.eq == SWP_EULER ? euler_batch_width(p, euler_cells) : width_for(p);
             if (n == 0) scheme = SWP_CLASSIC;   // N too small for any node width: classic items
         }
         if (scheme == SWP_SWEPT) {
@@ -1551,7 +1576,10 @@ swp_status tune_swept(const swp_desc* desc, const void* u0_host, int32_t count, 
 
 namespace swp {
 
-int swept_width(const swp_problem* p) { return width_for(p, true); }
+int swept_width(const swp_problem* p, int64_t euler_cells)
+{
+    return p->desc.eq == SWP_EULER ? euler_batch_width(p, euler_cells) : width_for(p, true);
+}
 
 int classic_chunk(const swp_problem* p) { return default_chunk(p); }
 

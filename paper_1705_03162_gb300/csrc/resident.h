@@ -4,6 +4,8 @@
 #pragma once
 
 #include <cstdint>
+#include <vector>
+
 #include <cuda_runtime.h>
 
 #include "scheme.cuh"
@@ -71,12 +73,19 @@ struct ResidentBatchWork {
     int* status;
     uint64_t wait_limit_ns;
 };
-int resident_batch_own(int esize);   // the most points a tile owns
-template <typename R> ResidentGeom resident_batch_geom(int eq, int bc, int64_t N, int64_t levels);
-template <typename R> int resident_batch_blocks(int sms);   // blocks resident at once
+struct ResidentBatchShape {
+    int variant = 0;       // of the kernel's tiles
+    int blocks = 0;        // resident at once
+};
+enum ResidentBatchFit { RESIDENT_FITS, RESIDENT_TOO_LONG, RESIDENT_SLOWER };
+// The tiles for problems of these sizes; TOO_LONG when some problem has more tiles
+// than the launch has blocks (or the launch cannot run), SLOWER when the dataflow
+// launch with its default widths is the faster form.
+ResidentBatchFit resident_batch_choose(int esize, const std::vector<int64_t>& points, int sms, ResidentBatchShape* out);
+ResidentGeom resident_batch_geom(int eq, int esize, int bc, int64_t N, int64_t levels, const ResidentBatchShape& s);
 template <typename R>
-cudaError_t launch_swept_resident_batch(const ResidentInst<R>* insts, const ResidentBatchWork& w, int blocks,
-                                        cudaStream_t s);
+cudaError_t launch_swept_resident_batch(const ResidentInst<R>* insts, const ResidentBatchWork& w,
+                                        const ResidentBatchShape& shape, cudaStream_t s);
 
 // The same for Euler (FP64): cells in shared memory, L levels per exchange, M = 1, P
 // = 1 where the interfaces' sides are tasks of their own, else 0; warps unused.

@@ -18,6 +18,7 @@
 // launch / this one: FP64, 400 to 1600 steps, 61.3 / 58.1 ms; FP32, 2000 to 10000
 // steps, 43.0 / 11.1 ms.
 #include <algorithm>
+#include <vector>
 
 #include "resident.h"
 #include "resident_tile.cuh"
@@ -26,26 +27,28 @@ namespace swp {
 
 namespace {
 
-// Points per thread, stale points at each end of a warp's round (edge = rad L),
-// rounds per exchange, and blocks, by precision: the fastest of a sweep on 256
-// heat and KS problems of 2^10..2^16 points.  Smaller blocks lose less at their
-// barriers when they share an SM (FP64, P = 12: 58.1 ms with 2 warps, 61.2 with 4,
-// 59.0 with 1, whose tiles have more halo); FP32 rounds stale whole lanes of
-// 16-point vectors (P = 16: 11.1 ms; 8: 12.4, 12: 11.6, 20: 11.2, 28: 11.4; KS runs
-// in pairs, which gain in the single launch, 12.2).
-template <typename R> struct Tile;
-template <> struct Tile<float> {
-    static constexpr int P = 16, EDGE = 16, M = 3, THREADS = 128, BLOCKS_PER_SM = 4;
-};
-template <> struct Tile<double> {
-    static constexpr int P = 12, EDGE = 4, M = 2, THREADS = 64, BLOCKS_PER_SM = 8;
+// Tiles: points per thread, stale points at each end of a warp's round (edge = rad
+// L), rounds per exchange, threads, and blocks per SM.  FP64 blocks have two warps:
+// smaller blocks lose less at their barriers when they share an SM (256 problems of
+// 2^10..2^16 points: 58.1 ms, 61.2 with four warps, 59.0 with one, whose tiles have
+// more halo).  FP32 rounds leave whole lanes of 8- or 16-point vectors stale.
+//
+// Long tiles do the least work beside their own points, short ones spread a small
+// batch over more of the chip (resident_batch_choose).
+template <typename R, int P_, int EDGE_, int M_, int THREADS_, int BLOCKS_PER_SM_> struct Tile {
+    using Real = R;
+    static constexpr int P = P_, EDGE = EDGE_, M = M_, THREADS = THREADS_, BLOCKS_PER_SM = BLOCKS_PER_SM_;
+    static constexpr int SLOTS = THREADS / 32 * (32 * P - 2 * EDGE) + 2 * EDGE;
+    static constexpr int HALO = EDGE * M;             // points per side of an exchange
+    static constexpr int OWN = SLOTS - 2 * HALO;      // the most points a tile owns
 };
 
-template <typename R>
-__global__ void __launch_bounds__(Tile<R>::THREADS, Tile<R>::BLOCKS_PER_SM)
-    swept_resident_batch_kernel(const ResidentInst<R>* insts, ResidentBatchWork w)
+template <typename T>
+__global__ void __launch_bounds__(T::THREADS, T::BLOCKS_PER_SM)
+    swept_resident_batch_kernel(const ResidentInst<typename T::Real>* insts, ResidentBatchWork w)
 {
-    constexpr int P = Tile<R>::P;
+    using R = typename T::Real;
+    constexpr int P = T::P;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int tile_s;
     for (;;) {
@@ -71,77 +74,128 @@ __global__ void __launch_bounds__(Tile<R>::THREADS, Tile<R>::BLOCKS_PER_SM)
     }
 }
 
-template <typename R>
-constexpr int kSlots = Tile<R>::THREADS / 32 * (32 * Tile<R>::P - 2 * Tile<R>::EDGE) + 2 * Tile<R>::EDGE;
-
-// Halo points per side of the widest exchange, and the most points a tile owns.
-template <typename R>
-constexpr int kHalo = Tile<R>::EDGE * Tile<R>::M;
-template <typename R>
-constexpr int kOwn = kSlots<R> - 2 * kHalo<R>;
-
-template <typename R>
-size_t batch_smem()
+struct Variant {
+    const void* kernel;
+    int P, edge, M, threads, blocks_per_sm, slots, halo, own;
+};
+template <typename T>
+Variant variant_of()
 {
-    return resident_smem((int)sizeof(R), Tile<R>::P, kSlots<R>, kHalo<R>);
+    return {(const void*)swept_resident_batch_kernel<T>, T::P, T::EDGE, T::M, T::THREADS, T::BLOCKS_PER_SM, T::SLOTS,
+            T::HALO, T::OWN};
 }
+
+// The variants of a precision, longest tiles first.
+const std::vector<Variant>& variants(int esize)
+{
+    static const std::vector<Variant> f32 = {variant_of<Tile<float, 16, 16, 3, 128, 4>>(),
+                                             variant_of<Tile<float, 8, 16, 3, 128, 4>>()};
+    static const std::vector<Variant> f64 = {
+        variant_of<Tile<double, 12, 4, 2, 64, 8>>(), variant_of<Tile<double, 6, 4, 2, 64, 8>>(),
+        variant_of<Tile<double, 4, 4, 4, 64, 8>>(), variant_of<Tile<double, 2, 4, 4, 64, 8>>()};
+    return esize == 4 ? f32 : f64;
+}
+
+size_t smem_of(int esize, const Variant& v) { return resident_smem(esize, v.P, v.slots, v.halo); }
 
 }  // namespace
 
-int resident_batch_own(int esize) { return esize == 4 ? kOwn<float> : kOwn<double>; }
-
-template <typename R>
-ResidentGeom resident_batch_geom(int eq, int bc, int64_t N, int64_t levels)
+// Measured, in ms, 300 to 1200 steps, P = 12 / 6 / 4 / 2 against the dataflow launch
+// with its default widths (points in all, FP64):
+//   4 problems,    22 k     4.36 / 2.35 / 1.54 / 0.88   1.82
+//   4 problems,    62 k     4.36 / 2.36 / 1.55 / 1.78   2.04
+//   16 problems,   90 k     5.24 / 2.85 / 2.56 / 2.78   2.51
+//   16 problems,  430 k     11.8 / 9.7 / 7.9 / 10.2     7.8
+//   48 problems,  270 k     7.1 / 8.0 / 6.8 / 4.7       4.3
+//   128 problems, 430 k     12.5 / 10.6 / 7.8 / 7.5     6.4
+//   48 problems,  740 k     17.6 / 12.0 / 9.1 / 11.7    9.4
+//   128 problems, 2.0 M     29.4 / 22.6 / 23.9 / 30.3   24.6
+//   256 problems, 4.0 M     58.3 / (P = 6 with 4-warp blocks 62.5)  61.3
+// A batch whose P = 2 tiles the chip holds three to a sub-partition takes the P that
+// keeps a level of its busiest sub-partition shortest; one of 2.8 waves of P = 4 tiles
+// or more the longest tiles that still make up waves enough to even out; in between
+// the dataflow launch is as fast or faster.  FP32 (P = 16 / 8, dataflow): 4 problems
+// 0.20 / 0.15 / 1.1, 128 problems of 2.0 M points 0.93 / 0.73 / 4.4, 256 of 4.0 M with
+// 2000 to 10000 steps 11.0 / 12.6 / 43.
+ResidentBatchFit resident_batch_choose(int esize, const std::vector<int64_t>& points, int sms, ResidentBatchShape* out)
 {
-    const int rad = eq == HEAT ? 1 : 2;
+    const auto& vs = variants(esize);
+    std::vector<int64_t> tiles(vs.size(), 0);
+    std::vector<bool> holds(vs.size(), true);   // no problem has more tiles than blocks
+    for (const int64_t N : points)
+        for (size_t i = 0; i < vs.size(); ++i) {
+            const int64_t K = (N + vs[i].own - 1) / vs[i].own;
+            tiles[i] += K;
+            holds[i] = holds[i] && K <= (int64_t)vs[i].blocks_per_sm * sms;
+        }
+    if (!holds[0]) return RESIDENT_TOO_LONG;
+    auto waves = [&](size_t i) { return (double)tiles[i] / ((double)vs[i].blocks_per_sm * sms); };
+    size_t pick = 0;
+    if (esize == 4) {
+        pick = waves(0) < 2.5 && holds[1] ? 1 : 0;
+    } else if (waves(3) <= 0.75) {
+        double best = 0.0;
+        for (size_t i = 0; i < vs.size(); ++i) {
+            const double warps = (double)tiles[i] * (vs[i].threads / 32) / (4.0 * sms);   // per sub-partition
+            const double level = vs[i].P * std::max(1.0, warps);
+            if (i == 0 || level < best) {
+                best = level;
+                pick = i;
+            }
+        }
+    } else if (waves(2) < 2.8) {
+        return RESIDENT_SLOWER;
+    } else {
+        pick = waves(0) >= 3.3 ? 0 : (waves(0) >= 1.5 ? 1 : 2);
+    }
+    while (pick > 0 && !holds[pick]) --pick;
+    out->variant = (int)pick;
+    const Variant& v = vs[out->variant];
+    const size_t smem = smem_of(esize, v);
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(v.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+        return RESIDENT_TOO_LONG;
+    int nb = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, v.kernel, v.threads, smem) != cudaSuccess ||
+        nb < v.blocks_per_sm)
+        return RESIDENT_TOO_LONG;
+    out->blocks = v.blocks_per_sm * sms;
+    return RESIDENT_FITS;
+}
+
+ResidentGeom resident_batch_geom(int eq, int esize, int bc, int64_t N, int64_t levels, const ResidentBatchShape& s)
+{
+    const Variant& v = variants(esize)[s.variant];
     ResidentGeom g{};
     g.N = N;
-    g.K = (int)((N + kOwn<R> - 1) / kOwn<R>);
-    g.L = Tile<R>::EDGE / rad;
-    g.E = g.L * Tile<R>::M;
-    g.h = kHalo<R>;
-    g.slots = kSlots<R>;
-    g.buf_elems = buffer_elems((int)sizeof(R), Tile<R>::P, kSlots<R>);
+    g.K = (int)((N + v.own - 1) / v.own);
+    g.L = v.edge / (eq == HEAT ? 1 : 2);
+    g.E = g.L * v.M;
+    g.h = v.halo;
+    g.slots = v.slots;
+    g.buf_elems = buffer_elems(esize, v.P, v.slots);
     g.pub = g.h + 1;
     g.cap = (int)std::min<int64_t>((N + g.K - 1) / g.K, 2 * g.pub);
     g.bc = bc;
     g.exchanges = (levels + g.E - 1) / g.E - 1;
     g.last = (int)(levels - g.exchanges * g.E);
-    g.parity_words = (int64_t)g.K * g.cap * (sizeof(R) == 8 ? 2 : 1);
+    g.parity_words = (int64_t)g.K * g.cap * (esize == 8 ? 2 : 1);
     return g;
 }
 
 template <typename R>
-int resident_batch_blocks(int sms)
+cudaError_t launch_swept_resident_batch(const ResidentInst<R>* insts, const ResidentBatchWork& w,
+                                        const ResidentBatchShape& shape, cudaStream_t s)
 {
-    const size_t smem = batch_smem<R>();
-    if (smem > 48 * 1024 && cudaFuncSetAttribute((const void*)swept_resident_batch_kernel<R>,
-                                                 cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return 0;
-    int nb = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, swept_resident_batch_kernel<R>, Tile<R>::THREADS,
-                                                      smem) !=
-        cudaSuccess)
-        return 0;
-    return nb * sms;
-}
-
-template <typename R>
-cudaError_t launch_swept_resident_batch(const ResidentInst<R>* insts, const ResidentBatchWork& w, int blocks,
-                                        cudaStream_t s)
-{
+    const Variant& v = variants((int)sizeof(R))[shape.variant];
     void* args[] = {(void*)&insts, (void*)&w};
-    return cudaLaunchCooperativeKernel((const void*)swept_resident_batch_kernel<R>, dim3((unsigned)blocks),
-                                       dim3(Tile<R>::THREADS), args, batch_smem<R>(), s);
+    return cudaLaunchCooperativeKernel(v.kernel, dim3((unsigned)std::min(shape.blocks, w.ntiles)),
+                                       dim3((unsigned)v.threads), args, smem_of((int)sizeof(R), v), s);
 }
 
-template ResidentGeom resident_batch_geom<double>(int, int, int64_t, int64_t);
-template ResidentGeom resident_batch_geom<float>(int, int, int64_t, int64_t);
-template int resident_batch_blocks<double>(int);
-template int resident_batch_blocks<float>(int);
-template cudaError_t launch_swept_resident_batch<double>(const ResidentInst<double>*, const ResidentBatchWork&, int,
-                                                         cudaStream_t);
-template cudaError_t launch_swept_resident_batch<float>(const ResidentInst<float>*, const ResidentBatchWork&, int,
-                                                        cudaStream_t);
+template cudaError_t launch_swept_resident_batch<double>(const ResidentInst<double>*, const ResidentBatchWork&,
+                                                         const ResidentBatchShape&, cudaStream_t);
+template cudaError_t launch_swept_resident_batch<float>(const ResidentInst<float>*, const ResidentBatchWork&,
+                                                        const ResidentBatchShape&, cudaStream_t);
 
 }  // namespace swp

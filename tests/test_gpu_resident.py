@@ -169,3 +169,29 @@ def test_batch_of_whole_advances(dtype):
     for (eq, bc, N, st), s, u, p in zip(cases, specs, u0, probs):
         assert np.array_equal(p.read(), _oracle(s, u, 4 * st)), (eq, bc, N, st)
         p.close()
+
+
+@pytest.mark.parametrize("dtype,count,lo,hi", [
+    ("f64", 1, 9001, 9002), ("f64", 5, 9000, 15000),            # short tiles
+    ("f64", 60, 5000, 6000),                                    # the dataflow launch, default widths
+    ("f64", 60, 15000, 16000), ("f64", 110, 15000, 16000), ("f64", 250, 15000, 16000),   # longer ones
+    ("f32", 3, 3000, 9000), ("f32", 220, 15000, 16000)])
+def test_batch_tile_lengths(dtype, count, lo, hi):
+    """Batches on each side of the lines between tile lengths, with widths that
+    the on-chip form does not use: every problem equals its classic advance."""
+    torch = pytest.importorskip("torch")
+    stream = torch.cuda.Stream()
+    rng = np.random.default_rng(count)
+    kinds = [("heat", "periodic"), ("ks", "periodic"), ("heat", "reflective")]
+    specs = [spec_for(*kinds[i % 3], int(rng.integers(lo, hi))) for i in range(count)]
+    steps = [int(rng.integers(17, 60)) for _ in specs]
+    u0 = [state_for(s, _np(dtype), seed=i) for i, s in enumerate(specs)]
+    probs = [S.Problem(s, u, dtype, stream=stream) for s, u in zip(specs, u0)]
+    with S.Batch(stream) as b:
+        b.advance_ex(probs, steps, ["swept"] * count, [S.fit_width(s.eq, s.n_points, 2048) for s in specs])
+        b.synchronize()
+    for s, u, st, p in zip(specs, u0, steps, probs):
+        with S.Problem(s, u, dtype, stream=stream) as q:
+            q.advance(st, "classic")
+            assert np.array_equal(p.read(), q.read()), (s.eq, s.bc, s.n_points, st)
+        p.close()
