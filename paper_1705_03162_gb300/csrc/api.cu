@@ -657,7 +657,10 @@ swp_status advance_typed(swp_problem* p, int64_t steps, const swp_advance_opts& 
     if (o.scheme == SWP_SCHEME_AUTO) {
         int n = 0;
         choice_for(p, &o.scheme, &n);
-        if (o.scheme == SWP_SWEPT && o.points_per_block == 0) o.points_per_block = n;
+        // a measured width; without one the default launch and width
+        Tuned t;
+        if (o.scheme == SWP_SWEPT && o.points_per_block == 0 && tuned_of(p->desc, &t) && t.n_swept > 0)
+            o.points_per_block = n;
     }
     if (o.scheme == SWP_SWEPT && o.points_per_block == 0 && o.launch != SWP_LAUNCH_REGISTER &&
         o.launch != SWP_LAUNCH_CLUSTER && default_width(p) == 0) {

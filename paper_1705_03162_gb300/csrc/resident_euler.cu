@@ -16,8 +16,8 @@
 // 152 SMs x 128 cells or fewer has one row each, where the swept form took
 // 2H - 1 dependent levels per H levels of progress.  Clocks (2.07 GHz) per level
 // against the dataflow launch, Sod / limited everywhere: N = 4096 8100 / 8200
-// (21200 / 22600 when this form came), 65536 22600 / 32900 (28000 / 48700), 200000
-// 56200 / 94700 (62200 / 115100).  Grids whose cells do not fit shared memory (N above about
+// (21200 / 22600 when this form came), 65536 22500 / 32700 (28000 / 48700), 200000
+// 54000 / 91000 (62200 / 115100).  Grids whose cells do not fit shared memory (N above about
 // 330000) keep that launch.
 //
 // Dirichlet ends: the tile's slots beyond an end hold that end's ghost state in
@@ -33,21 +33,27 @@ namespace swp {
 
 namespace {
 
-constexpr int kThreads = 256;
+// Threads per block: 16 warps hide the latencies that 8 leave at each sub-partition
+// (200000 cells limited everywhere: 91000 against 94800 clocks per level; 131072
+// cells, Sod: 36800 against 38200); a SPLIT tile has work for few warps (N = 4096: 8240
+// with 16, 8120 with 8).
+template <bool SPLIT>
+constexpr int kThreads = SPLIT ? 256 : 512;
 
 // SPLIT: for tiles of at most two rows of cells, whose passes would leave
 // sub-partitions idle: a cell's pressure and its sqrt(rho), and the two sides of
 // an interface, are tasks of their own on different warps (N = 4096: 8100 against
 // 10330 clocks per level).
 template <bool SPLIT>
-__global__ void __launch_bounds__(kThreads) swept_resident_euler_kernel(const double* A, double* B, ResidentGeom g,
+__global__ void __launch_bounds__(kThreads<SPLIT>) swept_resident_euler_kernel(const double* A, double* B, ResidentGeom g,
                                                                         Coefs<double> cp)
 {
     using R = double;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const Coefs<R> c = lane_coefs<R, EULER>(cp);
     const Units<R> ku = make_units<R, EULER>();
-    const int T = kThreads, tid = threadIdx.x;
+    constexpr int T = kThreads<SPLIT>;
+    const int tid = threadIdx.x;
     const int k = blockIdx.x, K = g.K, h = g.h, cap = g.cap, pub = g.pub;
     const int64_t N = g.N;
     const int64_t b0 = k * N / K;
@@ -262,7 +268,8 @@ cudaError_t launch_swept_resident_euler(int bc, const double* A, double* B, int6
     cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&A, (void*)&B, (void*)&g, (void*)&c};
-    return cudaLaunchCooperativeKernel(fn, dim3((unsigned)s.K), dim3(kThreads), args, smem, st);
+    return cudaLaunchCooperativeKernel(fn, dim3((unsigned)s.K), dim3(s.P ? kThreads<true> : kThreads<false>), args,
+                                       smem, st);
 }
 
 }  // namespace swp
