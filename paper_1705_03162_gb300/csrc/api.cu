@@ -267,7 +267,10 @@ int euler_batch_width(const swp_problem* p, int64_t cells)
 {
     Tuned t;
     if (tuned_of(p->desc, &t) && t.n_swept > 0 && check_width(p, t.n_swept) == SWP_OK) return t.n_swept;
-    const int64_t target = std::min(p->N / 2, std::max<int64_t>(64, std::min<int64_t>(512, cells / 1500)));
+    // (a short problem among large ones keeps some 48 nodes: its own chain of
+    // phases would outlast the rest)
+    const int64_t target =
+        std::min(p->N / 2, std::max<int64_t>(64, std::min<int64_t>(512, std::min(cells / 1500, p->N / 48))));
     for (int n = (int)(target / 8 * 8); n >= 8; n -= 8)
         if (check_width(p, n) == SWP_OK) return n;
     return 0;
@@ -431,8 +434,8 @@ bool run_swept_resident(swp_problem* p, int64_t steps, swp_status* st)
     if (!p->shape_known) {
         p->shape_known = true;
         const bool fits = p->desc.eq == SWP_EULER
-                              ? resident_euler_plan(p->N, p->sms, max_smem(p->device), &p->shape)
-                              : resident_plan(p->desc.eq, p->esize, p->N, p->sms, max_smem(p->device), &p->shape);
+                              ? resident_euler_plan(p->N, p->sms, &p->shape)
+                              : resident_plan(p->desc.eq, p->esize, p->N, p->sms, &p->shape);
         if (!fits) p->shape.K = 0;
     }
     if (p->shape.K == 0) return false;

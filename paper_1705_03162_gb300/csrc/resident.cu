@@ -146,7 +146,7 @@ double level_clocks(int eq, int esize, int warps, int P, int L, int M, int h)
 
 // The best shape for blocks that own `own` points each.  Returns its clocks per
 // level, 0 when no tile holds them.
-double best_shape(int eq, int esize, int own, size_t max_smem, ResidentShape* out)
+double best_shape(int eq, int esize, int own, ResidentShape* out)
 {
     const int rad = eq == HEAT ? 1 : 2;
     const int* pts = esize == 8 ? kPoints64 : kPoints32;
@@ -164,7 +164,7 @@ double best_shape(int eq, int esize, int own, size_t max_smem, ResidentShape* ou
                 const int M = std::min(64, (slots - own) / (2 * rad * L));
                 if (M < 1) continue;
                 const int h = rad * L * M;
-                if (resident_smem(esize, P, slots, h) > max_smem) continue;
+                if (resident_smem(esize, P, slots, h) > kResidentSmem) continue;
                 const double cost = level_clocks(eq, esize, warps, P, L, M, h);
                 if (best == 0.0 || cost < best) {
                     best = cost;
@@ -180,7 +180,7 @@ double best_shape(int eq, int esize, int own, size_t max_smem, ResidentShape* ou
 
 }  // namespace
 
-bool resident_plan(int eq, int esize, int64_t N, int sms, size_t max_smem, ResidentShape* out)
+bool resident_plan(int eq, int esize, int64_t N, int sms, ResidentShape* out)
 {
     *out = ResidentShape();
     if (eq == EULER || N < 64 || sms < 1) return false;
@@ -189,7 +189,7 @@ bool resident_plan(int eq, int esize, int64_t N, int sms, size_t max_smem, Resid
     const int K = (int)std::min<int64_t>(sms, std::max<int64_t>(1, N / 16));
     if ((N + 1) * (K + 1) < (int64_t)1 << 31) {
         const int own = (int)((N + K - 1) / K);
-        const double clocks = best_shape(eq, esize, own, max_smem, out);
+        const double clocks = best_shape(eq, esize, own, out);
         // FP64 from 2^17 points: the swept dataflow launch spends about 700
         // clocks per level above its points' pipe time (KS 2^17: 3760 against
         // 3965 here, 2^20: 25530 against 25930; heat 2^17: 1995 against 1690)
@@ -206,7 +206,7 @@ bool resident_plan(int eq, int esize, int64_t N, int sms, size_t max_smem, Resid
     const int64_t waves = (N + (int64_t)sms * 14000 - 1) / ((int64_t)sms * 14000);
     const int64_t blocks = waves * sms;
     if (blocks >= (int64_t)1 << 30) return false;
-    if (best_shape(eq, esize, (int)((N + blocks - 1) / blocks), max_smem, out) == 0.0) return false;
+    if (best_shape(eq, esize, (int)((N + blocks - 1) / blocks), out) == 0.0) return false;
     out->K = (int)blocks;
     out->waves = (int)std::min<int64_t>(waves, 1 << 20);
     return true;
@@ -250,10 +250,8 @@ cudaError_t launch_swept_resident(int eq, int bc, const R* A, R* B, int64_t N, i
     g.buf_elems = buffer_elems((int)sizeof(R), s.P, g.slots);
     const void* fn = kernel_of<R>(eq, s.P);
     if (!fn) return cudaErrorInvalidDeviceFunction;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    const cudaError_t e = allow_resident_smem(fn);
+    if (e != cudaSuccess) return e;
     void* args[] = {(void*)&A, (void*)&B, (void*)&g, (void*)&c};
     const dim3 grid((unsigned)s.K), block((unsigned)(32 * s.warps));
     return s.waves > 1 ? cudaLaunchKernel(fn, grid, block, args, smem, st)

@@ -12,6 +12,15 @@
 
 namespace swp {
 
+// Shared memory the resident kernels are allowed: always the same amount, so that
+// launches from several threads with tiles of different sizes cannot undo each
+// other's setting.
+constexpr size_t kResidentSmem = 226 * 1024;
+inline cudaError_t allow_resident_smem(const void* kernel)
+{
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kResidentSmem);
+}
+
 // One cooperative launch of K blocks, each keeping its part of the grid on chip.
 struct ResidentShape {
     int K = 0;        // blocks (0: N has no resident shape)
@@ -45,7 +54,7 @@ struct ResidentGeom {
     ResidentSync sync;
 };
 // The shape with the least estimated time per level, false when N does not fit.
-bool resident_plan(int eq, int esize, int64_t N, int sms, size_t max_smem, ResidentShape* out);
+bool resident_plan(int eq, int esize, int64_t N, int sms, ResidentShape* out);
 // 8-byte words of one parity, and exchanges of an advance of `levels` levels.
 size_t resident_words(int eq, int esize, int64_t N, const ResidentShape& s);
 int64_t resident_exchanges(const ResidentShape& s, int64_t levels);
@@ -89,7 +98,7 @@ cudaError_t launch_swept_resident_batch(const ResidentInst<R>* insts, const Resi
 
 // The same for Euler (FP64): cells in shared memory, L levels per exchange, M = 1, P
 // = 1 where the interfaces' sides are tasks of their own, else 0; warps unused.
-bool resident_euler_plan(int64_t N, int sms, size_t max_smem, ResidentShape* out);
+bool resident_euler_plan(int64_t N, int sms, ResidentShape* out);
 size_t resident_euler_words(int64_t N, const ResidentShape& s);
 cudaError_t launch_swept_resident_euler(int bc, const double* A, double* B, int64_t N, int64_t levels,
                                         const ResidentShape& s, const ResidentSync& y, const Coefs<double>& c,

@@ -152,9 +152,7 @@ ResidentBatchFit resident_batch_choose(int esize, const std::vector<int64_t>& po
     out->variant = (int)pick;
     const Variant& v = vs[out->variant];
     const size_t smem = smem_of(esize, v);
-    if (smem > 48 * 1024 &&
-        cudaFuncSetAttribute(v.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return RESIDENT_TOO_LONG;
+    if (allow_resident_smem(v.kernel) != cudaSuccess) return RESIDENT_TOO_LONG;
     int nb = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, v.kernel, v.threads, smem) != cudaSuccess ||
         nb < v.blocks_per_sm)

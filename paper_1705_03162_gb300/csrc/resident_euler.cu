@@ -207,7 +207,7 @@ int turns(int n) { return ((n + 31) / 32 + 3) / 4; }
 
 }  // namespace
 
-bool resident_euler_plan(int64_t N, int sms, size_t max_smem, ResidentShape* out)
+bool resident_euler_plan(int64_t N, int sms, ResidentShape* out)
 {
     *out = ResidentShape();
     if (N < 32 || sms < 1) return false;
@@ -218,7 +218,7 @@ bool resident_euler_plan(int64_t N, int sms, size_t max_smem, ResidentShape* out
     for (int split = 0; split < 2; ++split)
         for (int L = 2; L <= 48; L += 2) {
             const int W = own + 4 * L;
-            if (smem_of(own, L, split) > max_smem) break;
+            if (smem_of(own, L, split) > kResidentSmem) break;
             // FP64 operations of the passes (limited on some interfaces), their
             // barriers and latencies, and an exchange
             double clocks = 1700.0 + 20.0 * L;
@@ -265,7 +265,7 @@ cudaError_t launch_swept_resident_euler(int bc, const double* A, double* B, int6
     g.parity_words = (int64_t)resident_euler_words(N, s);
     const size_t smem = smem_of(own, s.L, s.P != 0);
     const void* fn = s.P ? (const void*)swept_resident_euler_kernel<true> : (const void*)swept_resident_euler_kernel<false>;
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const cudaError_t e = allow_resident_smem(fn);
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&A, (void*)&B, (void*)&g, (void*)&c};
     return cudaLaunchCooperativeKernel(fn, dim3((unsigned)s.K), dim3(s.P ? kThreads<true> : kThreads<false>), args,
