@@ -235,10 +235,10 @@ size_t swp_memory_in_use(void);
  * form where it is the faster one: a block keeps a tile of a problem for its
  * whole advance, the problem's tiles exchanging halos (one cooperative launch).
  * That is every FP32 group, and FP64 groups of few points (below about 80,000 in
- * all) or many (above about 750,000); FP64 groups in between run the table form
- * with its default widths.  In all these the given node widths are checked and
- * otherwise unused.  A problem with more tiles than the launch has blocks (about
- * 900,000 points) sends the group to the table form with the given widths.
+ * all); larger FP64 groups run the table form with node widths by their points in
+ * all (a tuned width that is not overridden stays).  In these the given node widths
+ * are checked and otherwise unused.  A problem above about 900,000 points sends the
+ * group to the table form with the given widths.
  * Each problem's result is bit-identical to swp_advance with the same scheme
  * (and, swept, the same node width).  The table costs 12 bytes of device
  * memory per (problem, phase) task, the on-chip form's halo words at most about

@@ -1209,10 +1209,41 @@ swp_status batch_launch(swp_batch* b, const std::vector<BatchItem>& items, std::
     return SWP_OK;
 }
 
+// Node width for N points from a target width w: N split into
+// K = max(2, ceil(N / w)) nearly equal nodes, the width a multiple of 4 rad,
+// so that the remainder widens some nodes by at most 4 rad and no node is
+// wider than w + 4 rad (a batch sizes its blocks for its widest node); 0 when
+// N has no two nodes of 4 rad points.
+int64_t fitted_width(int rad, int64_t N, int64_t w)
+{
+    const int64_t step = 4 * rad;
+    if (w < step || N < 2 * step) return 0;
+    const int64_t K = std::max<int64_t>(2, (N + w - 1) / w);
+    return std::max<int64_t>(step, (N / K) / step * step);
+}
+
+// Target node width of FP64 heat and KS problems of `points` points in all that
+// advance as whole advances in one dataflow launch: sqrt(points / 15), within 128 and
+// 2048.  Wide nodes have fewer phases, flags and halo loads per level; narrow ones
+// spread a batch over the chip and end together.  Measured, ms, nodes of 128 / 256 /
+// 512 / 1024 / 2048 points, 128 threads (and this rule's width):
+//   48 problems,   260 k points (132)   4.28 / 4.71 / 6.52 / 13.3 / 20.0
+//   48 problems,   720 k (219)          9.90 / 9.37 / 10.2 / 14.2 / 25.2
+//   128 problems,  2.1 M (374)          26.3 / 23.9 / 23.8 / 25.6 / 29.3
+//   256 problems,  3.9 M (507)          51.6 / 46.3 / 44.3 / 45.8 / 47.7
+//   512 problems,  7.7 M (715)          97.8 / 87.6 / 83.4 / 83.6 / 84.8
+//   4096 problems, 62.6 M (2043)           - /    - / 1218 / 1185 / 1168
+int64_t batch_width(int64_t points)
+{
+    return std::max<int64_t>(128, std::min<int64_t>(2048, (int64_t)std::sqrt((double)points / 15.0)));
+}
+// A problem above this is most of a batch's time by itself, and its widths stay.
+constexpr int64_t kLongProblem = 900000;
+
 // The batched resident launch of whole heat / KS advances (resident_batch.cu).
 // False (nothing launched) when the dataflow launch takes them: a problem has more
 // tiles than the launch has blocks, the launch cannot run cooperatively, or the
-// dataflow launch is faster, for which the plans get their default widths.
+// dataflow launch is faster, for which the plans get widths by the batch's size.
 constexpr int kFormResident = 100;   // batch_key form, beside the dataflow modes
 
 template <typename R>
@@ -1226,14 +1257,24 @@ bool resident_batch_group(swp_batch* b, std::vector<BatchItem>& plans, bool grap
     for (const auto& it : plans) points.push_back(it.p->N);
     ResidentBatchShape shape;
     const ResidentBatchFit fit = resident_batch_choose((int)sizeof(R), points, b->sms, &shape);
-    if (fit == RESIDENT_SLOWER)
+    if (fit == RESIDENT_SLOWER) {
+        int64_t total = 0, longest = 0;
+        for (const int64_t N : points) {
+            total += N;
+            longest = std::max(longest, N);
+        }
+        if (longest > kLongProblem) return false;
+        const int64_t target = batch_width(total);
         for (auto& it : plans) {
-            const int n = width_for(it.p);
-            if (n == 0 || n == it.s.n) continue;
+            Tuned t;   // (a width tuned for the problem, and not overridden, stays)
+            if (tuned_of(it.p->desc, &t) && t.n_swept == it.s.n) continue;
+            const int n = (int)fitted_width(it.p->rad, it.p->N, target);
+            if (n == 0 || n == it.s.n || check_width(it.p, n) != SWP_OK) continue;
             it.s = plan_swept(it.p, it.s.T / it.p->sub, n);
             it.p_hi = it.s.n_phases;
             it.flip = (it.s.top & 1) != 0;
         }
+    }
     if (fit != RESIDENT_FITS) return false;
     std::vector<BatchItem> items = plans;
     for (auto& it : items) it.flip = true;   // from one row to the other
@@ -1495,19 +1536,6 @@ swp_status batch_advance(swp_batch* b, swp_problem* const* problems, const int64
     if (threads < 0 || threads > max_threads || threads % 32)
         return fail(SWP_EINVAL, "threads must be 0 or a multiple of 32 in [32, %d]", max_threads);
     return launch_groups(b, groups, threads, launch == SWP_LAUNCH_GRAPH, true);
-}
-
-// Node width for N points from a target width w: N split into
-// K = max(2, ceil(N / w)) nearly equal nodes, the width a multiple of 4 rad,
-// so that the remainder widens some nodes by at most 4 rad and no node is
-// wider than w + 4 rad (a batch sizes its blocks for its widest node); 0 when
-// N has no two nodes of 4 rad points.
-int64_t fitted_width(int rad, int64_t N, int64_t w)
-{
-    const int64_t step = 4 * rad;
-    if (w < step || N < 2 * step) return 0;
-    const int64_t K = std::max<int64_t>(2, (N + w - 1) / w);
-    return std::max<int64_t>(step, (N / K) / step * step);
 }
 
 // Time two advances (the second timed) of `steps` timesteps of `count`

@@ -89,7 +89,7 @@ struct ResidentBatchShape {
 enum ResidentBatchFit { RESIDENT_FITS, RESIDENT_TOO_LONG, RESIDENT_SLOWER };
 // The tiles for problems of these sizes; TOO_LONG when some problem has more tiles
 // than the launch has blocks (or the launch cannot run), SLOWER when the dataflow
-// launch with its default widths is the faster form.
+// launch with widths by the batch's size is the faster form.
 ResidentBatchFit resident_batch_choose(int esize, const std::vector<int64_t>& points, int sms, ResidentBatchShape* out);
 ResidentGeom resident_batch_geom(int eq, int esize, int bc, int64_t N, int64_t levels, const ResidentBatchShape& s);
 template <typename R>

@@ -12,11 +12,10 @@
 // the end.  Several blocks share an SM: while one waits for its halos or a
 // barrier the others compute.
 //
-// What bounds it: the point updates' own pipe, FP64 (86 % of its peak with 4-warp
-// blocks, whose barriers lost the rest) or FP32 issue, plus the halos and the
-// tiles' unused slots.  256 heat and KS problems of 2^10..2^16 points, dataflow
-// launch / this one: FP64, 400 to 1600 steps, 61.3 / 58.1 ms; FP32, 2000 to 10000
-// steps, 43.0 / 11.1 ms.
+// What bounds it: FP32, instruction issue, plus the halos and the tiles' unused
+// slots: 256 heat and KS problems of 2^10..2^16 points, 2000 to 10000 steps, dataflow
+// launch 43.0 ms, this one 11.0.  FP64, for the batches that leave most of the chip
+// idle (resident_batch_choose), the levels' chains and exchanges.
 #include <algorithm>
 #include <vector>
 
@@ -29,9 +28,8 @@ namespace {
 
 // Tiles: points per thread, stale points at each end of a warp's round (edge = rad
 // L), rounds per exchange, threads, and blocks per SM.  FP64 blocks have two warps:
-// smaller blocks lose less at their barriers when they share an SM (256 problems of
-// 2^10..2^16 points: 58.1 ms, 61.2 with four warps, 59.0 with one, whose tiles have
-// more halo).  FP32 rounds leave whole lanes of 8- or 16-point vectors stale.
+// smaller blocks lose less at their barriers when they share an SM.  FP32 rounds
+// leave whole lanes of 8- or 16-point vectors stale.
 //
 // Long tiles do the least work beside their own points, short ones spread a small
 // batch over more of the chip (resident_batch_choose).
@@ -90,9 +88,8 @@ const std::vector<Variant>& variants(int esize)
 {
     static const std::vector<Variant> f32 = {variant_of<Tile<float, 16, 16, 3, 128, 4>>(),
                                              variant_of<Tile<float, 8, 16, 3, 128, 4>>()};
-    static const std::vector<Variant> f64 = {
-        variant_of<Tile<double, 12, 4, 2, 64, 8>>(), variant_of<Tile<double, 6, 4, 2, 64, 8>>(),
-        variant_of<Tile<double, 4, 4, 4, 64, 8>>(), variant_of<Tile<double, 2, 4, 4, 64, 8>>()};
+    static const std::vector<Variant> f64 = {variant_of<Tile<double, 4, 4, 4, 64, 8>>(),
+                                             variant_of<Tile<double, 2, 4, 4, 64, 8>>()};
     return esize == 4 ? f32 : f64;
 }
 
@@ -100,23 +97,21 @@ size_t smem_of(int esize, const Variant& v) { return resident_smem(esize, v.P, v
 
 }  // namespace
 
-// Measured, in ms, 300 to 1200 steps, P = 12 / 6 / 4 / 2 against the dataflow launch
-// with its default widths (points in all, FP64):
-//   4 problems,    22 k     4.36 / 2.35 / 1.54 / 0.88   1.82
-//   4 problems,    62 k     4.36 / 2.36 / 1.55 / 1.78   2.04
-//   16 problems,   90 k     5.24 / 2.85 / 2.56 / 2.78   2.51
-//   16 problems,  430 k     11.8 / 9.7 / 7.9 / 10.2     7.8
-//   48 problems,  270 k     7.1 / 8.0 / 6.8 / 4.7       4.3
-//   128 problems, 430 k     12.5 / 10.6 / 7.8 / 7.5     6.4
-//   48 problems,  740 k     17.6 / 12.0 / 9.1 / 11.7    9.4
-//   128 problems, 2.0 M     29.4 / 22.6 / 23.9 / 30.3   24.6
-//   256 problems, 4.0 M     58.3 / (P = 6 with 4-warp blocks 62.5)  61.3
-// A batch whose P = 2 tiles the chip holds three to a sub-partition takes the P that
-// keeps a level of its busiest sub-partition shortest; one of 2.8 waves of P = 4 tiles
-// or more the longest tiles that still make up waves enough to even out; in between
-// the dataflow launch is as fast or faster.  FP32 (P = 16 / 8, dataflow): 4 problems
-// 0.20 / 0.15 / 1.1, 128 problems of 2.0 M points 0.93 / 0.73 / 4.4, 256 of 4.0 M with
-// 2000 to 10000 steps 11.0 / 12.6 / 43.
+// FP64, in ms, 300 to 1200 steps, P = 4 / 2 against the dataflow launch with its best
+// node widths (points in all):
+//   4 problems,    22 k     1.54 / 0.88   1.8
+//   4 problems,    62 k     1.55 / 1.78   2.0
+//   16 problems,   90 k     2.56 / 2.78   2.5
+//   48 problems,  270 k      6.8 / 4.7    4.3
+// and with the longest tiles that still even out (P = 12 for the larger ones):
+//   48 problems,  1.2 M     17.7          15.4
+//   256 problems, 3.9 M     47.0          44.3
+//   4096 problems, 62.6 M   1290          1168
+// So a batch whose P = 2 tiles the chip holds three to a sub-partition runs on chip,
+// with the P that keeps a level of its busiest sub-partition shortest, and every other
+// one as dataflow.  FP32 (P = 16 / 8, dataflow): 4 problems 0.20 / 0.15 / 1.1, 128
+// problems of 2.0 M points 0.93 / 0.73 / 4.4, 256 of 4.0 M with 2000 to 10000 steps
+// 11.0 / 12.6 / 43.
 ResidentBatchFit resident_batch_choose(int esize, const std::vector<int64_t>& points, int sms, ResidentBatchShape* out)
 {
     const auto& vs = variants(esize);
@@ -128,27 +123,18 @@ ResidentBatchFit resident_batch_choose(int esize, const std::vector<int64_t>& po
             tiles[i] += K;
             holds[i] = holds[i] && K <= (int64_t)vs[i].blocks_per_sm * sms;
         }
-    if (!holds[0]) return RESIDENT_TOO_LONG;
     auto waves = [&](size_t i) { return (double)tiles[i] / ((double)vs[i].blocks_per_sm * sms); };
     size_t pick = 0;
     if (esize == 4) {
+        if (!holds[0]) return RESIDENT_TOO_LONG;
         pick = waves(0) < 2.5 && holds[1] ? 1 : 0;
-    } else if (waves(3) <= 0.75) {
-        double best = 0.0;
-        for (size_t i = 0; i < vs.size(); ++i) {
-            const double warps = (double)tiles[i] * (vs[i].threads / 32) / (4.0 * sms);   // per sub-partition
-            const double level = vs[i].P * std::max(1.0, warps);
-            if (i == 0 || level < best) {
-                best = level;
-                pick = i;
-            }
-        }
-    } else if (waves(2) < 2.8) {
-        return RESIDENT_SLOWER;
     } else {
-        pick = waves(0) >= 3.3 ? 0 : (waves(0) >= 1.5 ? 1 : 2);
+        if (waves(1) > 0.75) return RESIDENT_SLOWER;   // (below, every problem fits)
+        auto level = [&](size_t i) {
+            return vs[i].P * std::max(1.0, (double)tiles[i] * (vs[i].threads / 32) / (4.0 * sms));
+        };
+        pick = level(1) < level(0) ? 1 : 0;
     }
-    while (pick > 0 && !holds[pick]) --pick;
     out->variant = (int)pick;
     const Variant& v = vs[out->variant];
     const size_t smem = smem_of(esize, v);
