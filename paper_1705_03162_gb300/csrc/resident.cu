@@ -44,9 +44,9 @@
 // default before (cluster, Register and Shared graphs, per-phase FP32):
 //   heat FP64 N = 1024, 4096 steps      1196 -> 610 us
 //   heat FP64 reflective 50001, 2000    1559 -> 807 us
-//   KS FP64 10007, 2000 steps           3224 -> 1575 us
+//   KS FP64 10007, 2000 steps           3224 -> 1492 us
 //   heat FP32 2^17, 4000 steps          1080 -> 178 us
-//   KS FP32 2000003, 1000 steps         3710 -> 1014 us
+//   KS FP32 2000003, 1000 steps         3710 -> 1021 us
 #include <algorithm>
 
 #include "resident.h"

@@ -255,7 +255,7 @@ swp_status swp_server::round()
                               (rq->desc.n_points < ((int64_t)1 << (rq->desc.eq == SWP_EULER ? 13 : 17)) ||
                                rq->desc.dtype == SWP_F32);
     if (solo_phases) {
-        // as swp_advance would run it alone (SWP_LAUNCH_AUTO)
+        // per-phase launches: a range of phases cannot run on chip
         const swp::PhaseRange& r = ranges[0];
         const int64_t k0 = swp_kernel_launches(r.p);
         st = swp::advance_phases(r.p, r.n, r.steps, r.p_lo, r.p_hi);
