@@ -424,10 +424,25 @@ swp_status run_swept_persistent(swp_problem* p, const SweptPlan& s, int threads)
 // A test hook makes every wait of a launch wait for what is never published.
 uint32_t withheld_offset(const swp_problem* p) { return p->inject_withheld_flags ? (1u << 30) : 0u; }
 
+// Work captured from the stream may be replayed, each replay going on from the state
+// that the last one left.  (Also true when the status cannot be read.)
+bool capturing(cudaStream_t s)
+{
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) {
+        cudaGetLastError();
+        return true;
+    }
+    return cap != cudaStreamCaptureStatusNone;
+}
+
 // The resident form of the advance (resident.cu), where N has a shape for it.
 // Returns false (nothing done) when it has none, when the words cannot be allocated, or when
-// the stream is being captured: the sequence numbers are launch arguments, so
-// a replayed launch would accept the previous replay's words.
+// the stream is being captured.  A captured advance runs the forms whose state ends in
+// the row it began in (all but a heat advance of an odd number of levels), so that
+// replays go on from one another: here it ends in the other row, tiles of a larger
+// FP32 grid in either by their number of launches; and the sequence numbers are launch
+// arguments, so a replayed launch would accept the previous replay's words.
 template <typename R>
 bool run_swept_resident(swp_problem* p, int64_t steps, swp_status* st)
 {
@@ -438,7 +453,7 @@ bool run_swept_resident(swp_problem* p, int64_t steps, swp_status* st)
                               : resident_plan(p->desc.eq, p->esize, p->N, p->sms, &p->shape);
         if (!fits) p->shape.K = 0;
     }
-    if (p->shape.K == 0) return false;
+    if (p->shape.K == 0 || capturing(p->stream)) return false;
     const int64_t levels = steps * p->sub;
     if (p->shape.waves > 1) {
         const int64_t E = (int64_t)p->shape.L * p->shape.M;
@@ -456,12 +471,6 @@ bool run_swept_resident(swp_problem* p, int64_t steps, swp_status* st)
         *st = SWP_OK;
         return true;
     }
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(p->stream, &cap) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    if (cap != cudaStreamCaptureStatusNone) return false;
     const size_t bytes = 2 * sizeof(uint64_t) * (p->desc.eq == SWP_EULER
                                                      ? resident_euler_words(p->N, p->shape)
                                                      : resident_words(p->desc.eq, p->esize, p->N, p->shape));
