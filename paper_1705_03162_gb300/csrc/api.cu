@@ -1251,13 +1251,15 @@ constexpr int64_t kLongProblem = 900000;
 
 // The batched resident launch of whole heat / KS advances (resident_batch.cu).
 // False (nothing launched) when the dataflow launch takes them: a problem has more
-// tiles than the launch has blocks, the launch cannot run cooperatively, or the
-// dataflow launch is faster, for which the plans get widths by the batch's size.
+// tiles than the launch has blocks, the launch cannot run cooperatively, the stream is
+// being captured, or the dataflow launch is faster, for which the plans get widths by
+// the batch's size.
 constexpr int kFormResident = 100;   // batch_key form, beside the dataflow modes
 
 template <typename R>
 bool resident_batch_group(swp_batch* b, std::vector<BatchItem>& plans, bool graph, swp_status* st)
 {
+    if (capturing(b->stream)) return false;   // (it ends in the other row: see run_swept_resident)
     int coop = 0;
     if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, b->device) != cudaSuccess || !coop) return false;
     for (const auto& it : plans)

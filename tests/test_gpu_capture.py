@@ -40,3 +40,27 @@ def test_captured_tiled_advance_replays(eq, N, steps):
             for _ in range(3):
                 g.replay()
         assert np.array_equal(p.read(), _classic(spec, u0, "f32", 2 + 3 * steps))
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_captured_batch_advance_replays(dtype):
+    """A batch that runs on chip by default (from row to row), captured."""
+    torch = pytest.importorskip("torch")
+    specs = [spec_for("ks", "periodic", 3001), spec_for("heat", "periodic", 2000), spec_for("heat", "reflective", 777)]
+    u0 = [state_for(s, np.float64 if dtype == "f64" else np.float32, seed=i) for i, s in enumerate(specs)]
+    steps = [9, 10, 12]
+    stream = torch.cuda.Stream()
+    probs = [S.Problem(s, u, dtype, stream=stream) for s, u in zip(specs, u0)]
+    with S.Batch(stream) as b:
+        b.advance(probs, [2, 2, 2])
+        b.synchronize()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream, capture_error_mode="relaxed"):
+            b.advance_ex(probs, steps, ["swept"] * 3)
+        with torch.cuda.stream(stream):
+            for _ in range(3):
+                g.replay()
+        b.synchronize()
+        for s, u, st, p in zip(specs, u0, steps, probs):
+            assert np.array_equal(p.read(), _classic(s, u, dtype, 2 + 3 * st)), (s.eq, s.bc)
+            p.close()
