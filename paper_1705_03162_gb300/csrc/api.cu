@@ -436,6 +436,16 @@ bool capturing(cudaStream_t s)
     return cap != cudaStreamCaptureStatusNone;
 }
 
+// While it lives, this thread may allocate beside another thread's capture, which an
+// allocation in the default mode would fail under and break.
+struct RelaxedCapture {
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    ~RelaxedCapture() { cudaThreadExchangeStreamCaptureMode(&mode); }
+    RelaxedCapture(const RelaxedCapture&) = delete;
+    RelaxedCapture& operator=(const RelaxedCapture&) = delete;
+};
+
 // The resident form of the advance (resident.cu), where N has a shape for it.
 // Returns false (nothing done) when it has none, when the words cannot be allocated, or when
 // the stream is being captured.  A captured advance runs the forms whose state ends in
@@ -477,6 +487,7 @@ bool run_swept_resident(swp_problem* p, int64_t steps, swp_status* st)
     cudaError_t e = cudaSuccess;
     if (!p->words) {
         // the words, and the status word behind them
+        const RelaxedCapture relaxed;
         e = cudaMalloc((void**)&p->words, bytes + sizeof(int));
         if (e != cudaSuccess) {
             cudaGetLastError();

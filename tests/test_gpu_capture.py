@@ -1,5 +1,7 @@
 """Advances captured by the caller: each replay goes on from the state that the last
 one left, so a captured advance takes a form that ends in the row it began in."""
+import threading
+
 import numpy as np
 import pytest
 
@@ -64,3 +66,41 @@ def test_captured_batch_advance_replays(dtype):
         for s, u, st, p in zip(specs, u0, steps, probs):
             assert np.array_equal(p.read(), _classic(s, u, dtype, 2 + 3 * st)), (s.eq, s.bc)
             p.close()
+
+
+@pytest.mark.parametrize("eq,bc,N,dtype", [("heat", "periodic", 1024, "f64"), ("ks", "periodic", 2048, "f32"),
+                                           ("euler", "dirichlet", 300, "f64")])
+def test_first_advance_beside_another_threads_capture(eq, bc, N, dtype):
+    """A problem's first default advance (it allocates its halo words) while
+    another thread captures its own stream: both go through."""
+    torch = pytest.importorskip("torch")
+    spec = spec_for(eq, bc, N)
+    u0 = state_for(spec, np.float64 if dtype == "f64" else np.float32)
+    begun, done, out = threading.Event(), threading.Event(), []
+
+    def capture():
+        try:
+            x = torch.zeros(8, device="cuda")
+            g = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(g, stream=torch.cuda.Stream()):   # the default: global mode
+                x += 1
+                begun.set()
+                done.wait(30)
+            g.replay()
+            torch.cuda.synchronize()
+            out.append(float(x[0]))
+        finally:
+            begun.set()
+
+    with S.Problem(spec, u0, dtype, stream=torch.cuda.Stream()) as p:
+        th = threading.Thread(target=capture)
+        th.start()
+        try:
+            assert begun.wait(30)
+            p.advance(20, "swept")
+        finally:
+            done.set()
+            th.join()
+        assert out == [1.0]
+        assert p.kernel_launches() == 1
+        assert np.array_equal(p.read(), _classic(spec, u0, dtype, 20))
