@@ -57,7 +57,7 @@ struct swp_problem {
     bool shape_known = false;
     ResidentShape shape;
     uint64_t* words = nullptr;
-    int* resident_status = nullptr;   // status word of resident launches, once one has run
+    int* resident_status = nullptr;   // their status word: mapped host memory, so that reading it costs no copy
     uint32_t seq = 1;
 };
 
@@ -486,15 +486,22 @@ bool run_swept_resident(swp_problem* p, int64_t steps, swp_status* st)
                                                      : resident_words(p->desc.eq, p->esize, p->N, p->shape));
     cudaError_t e = cudaSuccess;
     if (!p->words) {
-        // the words, and the status word behind them
         const RelaxedCapture relaxed;
-        e = cudaMalloc((void**)&p->words, bytes + sizeof(int));
+        if (!p->resident_status &&
+            cudaHostAlloc((void**)&p->resident_status, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) !=
+                cudaSuccess) {
+            cudaGetLastError();
+            p->resident_status = nullptr;
+            return false;
+        }
+        *p->resident_status = 0;
+        e = cudaMalloc((void**)&p->words, bytes);
         if (e != cudaSuccess) {
             cudaGetLastError();
             p->words = nullptr;
             return false;
         }
-        e = cudaMemsetAsync(p->words, 0, bytes + sizeof(int), p->stream);
+        e = cudaMemsetAsync(p->words, 0, bytes, p->stream);
         p->seq = 1;
     }
     const int64_t exchanges = resident_exchanges(p->shape, levels);
@@ -513,7 +520,7 @@ bool run_swept_resident(swp_problem* p, int64_t steps, swp_status* st)
     y.seq = p->seq;
     y.wait_offset = withheld_offset(p);
     y.wait_limit_ns = p->wait_limit_ns;
-    y.status = (int*)((char*)p->words + bytes);
+    y.status = p->resident_status;
     if (p->desc.eq == SWP_EULER)
         e = launch_swept_resident_euler(p->desc.bc, (const double*)p->rows[p->cur], (double*)p->rows[1 - p->cur], p->N,
                                         levels, p->shape, y, coefs_of<double>(p), p->stream);
@@ -526,24 +533,29 @@ bool run_swept_resident(swp_problem* p, int64_t steps, swp_status* st)
         return false;
     }
     p->launches++;
-    p->resident_status = y.status;
     p->seq += (uint32_t)exchanges;
     *st = e == cudaSuccess ? SWP_OK : cuda_fail(e, "resident swept launch");
     if (e == cudaSuccess) p->cur = 1 - p->cur;
     return true;
 }
 
-// Reads the device status word of persistent launches (stream must be idle).
+// Reads the status words of persistent and resident launches (stream must be idle).
 swp_status check_device_status(swp_problem* p)
 {
     bool gave_up = false;
-    for (int* word : {p->status, p->resident_status}) {
-        if (!word) continue;
+    if (p->status) {
         int st = 0;
-        cudaError_t e = cudaMemcpy(&st, word, sizeof(int), cudaMemcpyDeviceToHost);
+        cudaError_t e = cudaMemcpy(&st, p->status, sizeof(int), cudaMemcpyDeviceToHost);
         if (e != cudaSuccess) return cuda_fail(e, "status read");
         if (st != 0) {
-            cudaMemset(word, 0, sizeof(int));
+            cudaMemset(p->status, 0, sizeof(int));
+            gave_up = true;
+        }
+    }
+    if (p->resident_status) {
+        volatile int* st = p->resident_status;
+        if (*st != 0) {
+            *st = 0;
             gave_up = true;
         }
     }
@@ -943,6 +955,7 @@ swp_status swp_destroy(swp_problem* p)
     if (p->batch) swp_batch_destroy(p->batch);
     if (p->status) cudaFree(p->status);
     if (p->words) cudaFree(p->words);
+    if (p->resident_status) cudaFreeHost(p->resident_status);
     for (auto& g : p->graphs) cudaGraphExecDestroy(g.exec);
     if (p->capture_stream) cudaStreamDestroy(p->capture_stream);
     g_in_use -= p->bytes;
