@@ -94,8 +94,8 @@ NCU_TRAFFIC = {
 # Issue-slot use of the batched FP32 launch from one ncu capture (the 4096
 # instances of the batched workload; the on-chip tiles of resident_batch.cu): warp
 # instructions issued over 4 per SM per cycle, keyed like the traffic record
-# and reported when the timed batch runs that width.
-NCU_ISSUE_FP32_BATCH = {"src": "b90796f1a92fd58a", "width": 2048, "issue_frac": 0.715, "issue_active": 0.715,
+# and reported when the timed batch runs on chip.
+NCU_ISSUE_FP32_BATCH = {"src": "b90796f1a92fd58a", "form": "on chip", "issue_frac": 0.715, "issue_active": 0.715,
                         "fma_pipe": 0.635}
 KERNEL_OF_LAUNCH = {"per_phase": "swept_phase_kernel", "graph": "swept_phase_kernel",
                     "persistent": "swept_batch_kernel", "auto": "swept_batch_kernel"}
@@ -333,12 +333,14 @@ def run_batched(count: int = 4096, seed: int = 20170509, dtypes=("f64", "f32"), 
     """4096 independent heat + KS instances (batched_cases), one persistent
     launch per precision replayed from a CUDA graph, against advancing a
     sample of the same instances one by one, whose results must equal the
-    batch's bit for bit.  Node widths (or `width` for every instance): the
-    fastest, on one advance of the whole batch, of the library autotuner's
-    choice per (equation, nearest power-of-two N) bucket and of one width for
+    batch's bit for bit.  The plan is the fastest, on one advance of the whole
+    batch, of the library's own choice (on chip, or the table form with widths
+    by the batch's size) and of the table form with the library autotuner's
+    choice per (equation, nearest power-of-two N) bucket or with one width for
     every instance (256, 512, 1024, 2048), each fitted to N (fit_width).  The
     autotuner measures each bucket alone; in the mixed batch every block is
-    sized for the widest node, which can change the order."""
+    sized for the widest node, which can change the order.  `width`: the
+    library's own choice with this width given."""
     import torch
     from paper_1705_03162_gb300 import swept as S
     cases = batched_cases(count, seed)
@@ -355,7 +357,10 @@ def run_batched(count: int = 4096, seed: int = 20170509, dtypes=("f64", "f32"), 
             probs.append(S.Problem(spec, u0, dtype, stream=stream))
 
         def assign(choice):
-            """(schemes, widths) of a candidate: a bucket table or one width."""
+            """(schemes, widths) of a candidate: a bucket table, one width, or
+            None for the library's choice."""
+            if choice is None:
+                return ["swept"] * len(cases), None
             sc, wd = [], []
             for eq, N, _ in cases:
                 scheme, n = choice[(eq, bucket(N))] if isinstance(choice, dict) else ("swept", choice)
@@ -366,7 +371,7 @@ def run_batched(count: int = 4096, seed: int = 20170509, dtypes=("f64", "f32"), 
         def advance_ms(sc, wd, bt):
             ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             ev0.record(stream)
-            bt.advance_ex(probs, steps, sc, wd, threads=threads, launch="persistent")
+            bt.advance_ex(probs, steps, sc, wd, threads=threads, launch="auto" if wd is None else "persistent")
             ev1.record(stream)
             ev1.synchronize()
             return ev0.elapsed_time(ev1)
@@ -388,30 +393,40 @@ def run_batched(count: int = 4096, seed: int = 20170509, dtypes=("f64", "f32"), 
                 # one width for every instance, fitted to each N, timed by the
                 # library on the batch itself (states put back after each)
                 _, best_u, ms_u = bt.tune_width(probs, steps, uniform, threads=threads)
-                # and the per-bucket autotuner's choice, timed the same way
+                # and the per-bucket autotuner's choice and the library's, timed the same way
                 ms_b = advance_ms(*assign(tuned), bt)
+                ms_l = advance_ms(*assign(None), bt)
             for p, (_, u0) in zip(probs, inputs):   # back to the initial states
                 p.write(u0)
-            times = {"per-bucket autotune": ms_b, **{str(w): m for w, m in zip(uniform, ms_u)}}
+            times = {"library": ms_l, "per-bucket autotune": ms_b, **{str(w): m for w, m in zip(uniform, ms_u)}}
             tuning["one_advance_ms"] = {k: round(v, 2) for k, v in times.items()}
             chosen = tuned if ms_b < ms_u[best_u] else uniform[best_u]
-            tuning["chosen"] = "per-bucket autotune" if isinstance(chosen, dict) else str(chosen)
+            if ms_l <= min(times.values()):
+                chosen = None
+            tuning["chosen"] = ("library" if chosen is None else
+                                "per-bucket autotune" if isinstance(chosen, dict) else str(chosen))
         tune_s = time.perf_counter() - t0
         schemes, widths = assign(chosen)
+        # a table's widths hold in a graph with a given block size (here the default one)
+        if not width and chosen is not None and not threads:
+            threads_run = 32 if dtype == "f32" else 128
+        else:
+            threads_run = threads
         with S.Batch(stream) as bt:
             # warm-up: two advances captured as CUDA graphs (an instance whose
             # advance ends in its other row alternates between two); the timed
             # third advance replays the first graph
             for _ in range(2):
-                bt.advance_ex(probs, steps, schemes, widths, threads=threads, launch="graph")
+                bt.advance_ex(probs, steps, schemes, widths, threads=threads_run, launch="graph")
             bt.synchronize()
             l0 = bt.kernel_launches()
             ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
             ev0.record(stream)
-            bt.advance_ex(probs, steps, schemes, widths, threads=threads, launch="graph")
+            bt.advance_ex(probs, steps, schemes, widths, threads=threads_run, launch="graph")
             ev1.record(stream)
             bt.synchronize()
             ms = ev0.elapsed_time(ev1)
+            on_chip = bt.debug_form()[0]
             launches = bt.kernel_launches() - l0
         # a sample advanced one problem at a time (the first advance timed),
         # the sample advanced one by one with the library defaults (scheme,
@@ -441,11 +456,12 @@ def run_batched(count: int = 4096, seed: int = 20170509, dtypes=("f64", "f32"), 
         ops = sum(c[1] * c[2] * op_count(c[0], "ops") for c in cases)
         peak = FP32_PEAK_TFLOPS if dtype == "f32" else FP64_PEAK_TFLOPS
         out[dtype] = {"value": upd / ms / 1e6, "unit": UNIT, "ms": ms, "kernel_launches": launches,
-                      "launch": "persistent kernel replayed from a CUDA graph",
+                      "launch": f"{'on-chip' if on_chip else 'persistent'} kernel replayed from a CUDA graph",
                       "per_instance_value": su / solo_s / 1e9, "autotune_s": tune_s,
                       "swept_instances": sum(1 for x in schemes if x == "swept"),
-                      "instances_with_wider_nodes": sum(1 for (e, N, _), sc, n in zip(cases, schemes, widths)
-                                                        if sc == "swept" and N % n),
+                      "instances_on_chip": on_chip,
+                      "instances_with_wider_nodes": None if on_chip or widths is None else
+                      sum(1 for (e, N, _), sc, n in zip(cases, schemes, widths) if sc == "swept" and N % n),
                       "sample_equals_solo_bitwise": f"{len(sample)} of {count} instances",
                       "roofline": {"bound": "alu", "achieved": flops / ms / 1e9, "peak": peak, "unit": "TFLOP/s",
                                    "frac": flops / ms / 1e9 / peak, "pipe_ops_frac": ops / ms / 1e9 / (peak / 2),
@@ -453,9 +469,9 @@ def run_batched(count: int = 4096, seed: int = 20170509, dtypes=("f64", "f32"), 
                                             f"({eqs.count('heat')} heat, {eqs.count('ks')} KS)",
                                    "peak_note": f"measured {'FP32' if dtype == 'f32' else 'FP64'} pipe",
                                    "issue": (dict(NCU_ISSUE_FP32_BATCH, bound="issue",
-                                                  note="ncu capture of this workload at that width")
+                                                  note="ncu capture of this workload in that form")
                                              if dtype == "f32" and NCU_ISSUE_FP32_BATCH["src"] == _kernel_src_hash()
-                                             and chosen == NCU_ISSUE_FP32_BATCH["width"] else None)},
+                                             and on_chip == count else None)},
                       "widths": tuning if tuning else f"every instance {width}, fitted to N"}
     return out
 
@@ -970,8 +986,9 @@ def main():
                          "fix the swept configuration")
     ap.add_argument("--batched", type=int, metavar="COUNT",
                     help="print the batched heat+KS line for COUNT instances in the --dtype precision instead; "
-                         "--points-per-block, when given, replaces the autotuned widths, and --threads sets "
-                         "the batch's block size")
+                         "--points-per-block, when given, skips the tuning and gives every problem this width "
+                         "(the library's own form and widths hold all the same, unless --threads sets "
+                         "the batch's block size)")
     ap.add_argument("--served", type=int, metavar="COUNT", help="print the served line for COUNT requests instead")
     ap.add_argument("--other", choices=["heat", "sod"], nargs="+",
                     help="print the heat-configuration and / or Sod line instead")

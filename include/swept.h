@@ -237,8 +237,10 @@ size_t swp_memory_in_use(void);
  * That is every FP32 group, and FP64 groups of few points (below about 80,000 in
  * all); larger FP64 groups run the table form with node widths by their points in
  * all (a tuned width that is not overridden stays).  In these the given node widths
- * are checked and otherwise unused.  A problem above about 900,000 points sends the
- * group to the table form with the given widths.
+ * are checked and otherwise unused; they hold with SWP_LAUNCH_PERSISTENT (always the
+ * table form) and with a given block size.  A problem above about 1,100,000 points
+ * (FP32) or 900,000 (FP64, in a group too large for the on-chip form) sends the group
+ * to the table form with the given widths.
  * Each problem's result is bit-identical to swp_advance with the same scheme
  * (and, swept, the same node width).  The table costs 12 bytes of device
  * memory per (problem, phase) task, the on-chip form's halo words at most about
@@ -269,8 +271,10 @@ swp_status swp_batch_advance(swp_batch* b, swp_problem* const* problems, const i
  *                      per problem; NULL or 0 = the tuned width, else the
  *                      default (classic: min(N, 1024), Euler min(N, 256);
  *                      swept as for swp_batch_advance)
- *   launch           : SWP_LAUNCH_AUTO or _PERSISTENT (upload the task table
- *                      and launch), or SWP_LAUNCH_GRAPH: the launch is
+ *   launch           : SWP_LAUNCH_AUTO (upload the tables and launch),
+ *                      SWP_LAUNCH_PERSISTENT (the same, always in the table
+ *                      form, where the given widths hold), or
+ *                      SWP_LAUNCH_GRAPH: AUTO's launch
  *                      captured as a CUDA graph with tables of its own on the
  *                      first advance of these problems, in their current
  *                      rows, with these plans, and replayed when the same
@@ -321,10 +325,12 @@ swp_status swp_fit_width(int32_t eq, int64_t n_points, int32_t target, int32_t* 
  * the n_candidates target widths, every problem's width is fitted to its N
  * (swp_fit_width; 0, the default rule, where the fitted width is not valid
  * for the problem) and problems[0..count) are advanced once by n_steps[i]
- * (swept, one persistent launch per group, block size `threads` as for
- * swp_batch_advance), timed with CUDA events on the batch's stream (the
- * span includes the host building and uploading the task tables, as a
- * plain advance would).  A problem listed twice is rejected by the advance
+ * (swept, SWP_LAUNCH_PERSISTENT: the table form with exactly these widths, block
+ * size `threads` as for swp_batch_advance), timed with CUDA events on the batch's
+ * stream (the span includes the host building and uploading the task tables, as a
+ * plain advance would).  Run the chosen widths with SWP_LAUNCH_PERSISTENT or the same
+ * given block size: SWP_LAUNCH_AUTO and _GRAPH with the default block size choose form
+ * and widths themselves, mostly the faster way.  A problem listed twice is rejected by the advance
  * (SWP_EINVAL) after the states are saved, and put back.  The
  * fastest candidate's per-problem widths are written to widths_out[count],
  * its index to *best (may be NULL), and each candidate's milliseconds to
@@ -402,6 +408,10 @@ swp_status swp_server_destroy(swp_server* s);
  * or hangs.  The paper has no counterpart: its nodes synchronise only at
  * kernel boundaries (Section 3). */
 swp_status swp_debug_withhold_flags(swp_problem* p, int withhold, int64_t wait_limit_ns);
+
+/* For tests: what form the batch's last advance took.  *on_chip: problems that ran
+ * in the on-chip form; *nodes: nodes (classic: chunks) of those in the table form. */
+swp_status swp_debug_batch_form(const swp_batch* b, int64_t* on_chip, int64_t* nodes);
 
 /* Swept advance that allocates nothing.  The paper has no counterpart: it is
  * here for callers that cannot call cudaMalloc -- code whose device memory is

@@ -1051,6 +1051,7 @@ struct swp_batch {
     std::vector<BatchGraph> graphs;    // at most 8, oldest first
     cudaStream_t capture_stream = nullptr;
     uint64_t wait_limit_ns = 2000000000ull;
+    int64_t on_chip = 0, nodes = 0;    // of the last advance: problems on chip, nodes and chunks of the table form
 };
 
 namespace {
@@ -1083,6 +1084,7 @@ struct BatchItem {
     SweptPlan s;    // swept plan; classic: n = widest chunk, K = chunks, n_phases = sub-steps
     int64_t p_lo, p_hi;   // phases of the plan this launch runs
     bool flip;      // the state ends in the other row (the plan's last phase runs)
+    bool given = false;   // the caller gave the node width
 };
 
 // Classic instance of a batch: K = ceil(N / m) chunks of the balanced
@@ -1277,11 +1279,12 @@ constexpr int64_t kLongProblem = 900000;
 // False (nothing launched) when the dataflow launch takes them: a problem has more
 // tiles than the launch has blocks, the launch cannot run cooperatively, the stream is
 // being captured, or the dataflow launch is faster, for which the plans get widths by
-// the batch's size.
+// the batch's size.  table: the caller asks for the dataflow launch, where the widths
+// that it gave hold.
 constexpr int kFormResident = 100;   // batch_key form, beside the dataflow modes
 
 template <typename R>
-bool resident_batch_group(swp_batch* b, std::vector<BatchItem>& plans, bool graph, swp_status* st)
+bool resident_batch_group(swp_batch* b, std::vector<BatchItem>& plans, bool table, bool graph, swp_status* st)
 {
     if (capturing(b->stream)) return false;   // (it ends in the other row: see run_swept_resident)
     int coop = 0;
@@ -1301,6 +1304,7 @@ bool resident_batch_group(swp_batch* b, std::vector<BatchItem>& plans, bool grap
         if (longest > kLongProblem) return false;
         const int64_t target = batch_width(total);
         for (auto& it : plans) {
+            if (table && it.given) continue;
             Tuned t;   // (a width tuned for the problem, and not overridden, stays)
             if (tuned_of(it.p->desc, &t) && t.n_swept == it.s.n) continue;
             const int n = (int)fitted_width(it.p->rad, it.p->N, target);
@@ -1310,7 +1314,7 @@ bool resident_batch_group(swp_batch* b, std::vector<BatchItem>& plans, bool grap
             it.flip = (it.s.top & 1) != 0;
         }
     }
-    if (fit != RESIDENT_FITS) return false;
+    if (fit != RESIDENT_FITS || table) return false;
     std::vector<BatchItem> items = plans;
     for (auto& it : items) it.flip = true;   // from one row to the other
     std::vector<int64_t> key;
@@ -1483,18 +1487,22 @@ swp_status persistent_via_batch(swp_problem* p, const SweptPlan& s, int threads)
 }
 
 // One group launch per (equation group, dtype) of the given items.
-// whole: the items are whole advances (not ranges of open ones).
-swp_status launch_groups(swp_batch* b, std::vector<BatchItem> (&groups)[2][2], int threads, bool graph, bool whole)
+// whole: the items are whole advances (not ranges of open ones).  table: no on-chip
+// form.
+swp_status launch_groups(swp_batch* b, std::vector<BatchItem> (&groups)[2][2], int threads, bool graph, bool whole,
+                         bool table)
 {
+    b->on_chip = b->nodes = 0;
     for (int g = 0; g < 2; ++g)
         for (int dt = 0; dt < 2; ++dt) {
             if (groups[g][dt].empty()) continue;
             const int mode = g == 1 ? SWP_EULER : SWP_HEAT;
             swp_status rs = SWP_OK;
             if (whole && g == 0 && threads == 0 &&
-                (dt == SWP_F64 ? resident_batch_group<double>(b, groups[g][dt], graph, &rs)
-                               : resident_batch_group<float>(b, groups[g][dt], graph, &rs))) {
+                (dt == SWP_F64 ? resident_batch_group<double>(b, groups[g][dt], table, graph, &rs)
+                               : resident_batch_group<float>(b, groups[g][dt], table, graph, &rs))) {
                 if (rs != SWP_OK) return rs;
+                b->on_chip += (int64_t)groups[g][dt].size();
                 continue;
             }
             // default block, measured on the batched heat+KS workload: 128
@@ -1505,6 +1513,7 @@ swp_status launch_groups(swp_batch* b, std::vector<BatchItem> (&groups)[2][2], i
             swp_status st = dt == SWP_F64 ? batch_group<double>(b, groups[g][dt], mode, thr, graph)
                                           : batch_group<float>(b, groups[g][dt], mode, thr, graph);
             if (st != SWP_OK) return st;
+            for (const auto& it : groups[g][dt]) b->nodes += it.s.K;
         }
     return SWP_OK;
 }
@@ -1538,6 +1547,7 @@ swp_status batch_advance(swp_batch* b, swp_problem* const* problems, const int64
             return fail(SWP_EINVAL, "unknown scheme %d for problem %d", scheme, i);
         if (n_steps[i] == 0) continue;
         int n = points_per_block ? points_per_block[i] : 0;
+        const bool given = n != 0;
         if (scheme == SWP_SCHEME_AUTO) {
             int tn = 0;
             choice_for(p, &scheme, &tn);
@@ -1545,6 +1555,7 @@ swp_status batch_advance(swp_batch* b, swp_problem* const* problems, const int64
         }
         BatchItem it;
         it.p = p;
+        it.given = given;
         if (scheme == SWP_SWEPT && n == 0) {
             n = p->desc.eq == SWP_EULER ? euler_batch_width(p, euler_cells) : width_for(p);
             if (n == 0) scheme = SWP_CLASSIC;   // N too small for any node width: classic items
@@ -1570,7 +1581,7 @@ swp_status batch_advance(swp_batch* b, swp_problem* const* problems, const int64
     }
     if (threads < 0 || threads > max_threads || threads % 32)
         return fail(SWP_EINVAL, "threads must be 0 or a multiple of 32 in [32, %d]", max_threads);
-    return launch_groups(b, groups, threads, launch == SWP_LAUNCH_GRAPH, true);
+    return launch_groups(b, groups, threads, launch == SWP_LAUNCH_GRAPH, true, launch == SWP_LAUNCH_PERSISTENT);
 }
 
 // Time two advances (the second timed) of `steps` timesteps of `count`
@@ -1685,7 +1696,7 @@ swp_status batch_advance_phases(swp_batch* b, const PhaseRange* ranges, int coun
                   (classic ? (p->desc.eq == SWP_HEAT && (it.s.T & 1)) : (it.s.top & 1) != 0);
         groups[p->desc.eq == SWP_EULER ? 1 : 0][p->desc.dtype].push_back(it);
     }
-    return launch_groups(b, groups, threads, false, false);
+    return launch_groups(b, groups, threads, false, false, true);
 }
 
 swp_status set_error(swp_status s, const char* msg) { return fail(s, "%s", msg); }
@@ -1785,6 +1796,14 @@ swp_status swp_batch_destroy(swp_batch* b)
 }
 
 int64_t swp_batch_kernel_launches(const swp_batch* b) { return b ? b->launches : -1; }
+
+swp_status swp_debug_batch_form(const swp_batch* b, int64_t* on_chip, int64_t* nodes)
+{
+    if (!b || !on_chip || !nodes) return fail(SWP_EINVAL, "batch, on_chip or nodes is NULL");
+    *on_chip = b->on_chip;
+    *nodes = b->nodes;
+    return SWP_OK;
+}
 
 swp_status swp_autotune_width(const swp_desc* desc, const void* u0_host, int32_t batch_count,
                               int64_t steps, int32_t* best_n)

@@ -44,7 +44,7 @@ ABI_SYMBOLS = (
     "swp_batch_kernel_launches", "swp_autotune_width", "swp_tuned_width",
     "swp_batch_advance_ex", "swp_autotune", "swp_tuned", "swp_fit_width", "swp_batch_tune_width",
     "swp_server_create", "swp_server_submit", "swp_server_poll", "swp_server_wait",
-    "swp_server_stats", "swp_server_destroy",
+    "swp_server_stats", "swp_server_destroy", "swp_debug_batch_form",
 )
 
 
@@ -126,6 +126,7 @@ def load_library(path: str = LIB_PATH):
             "swp_batch_synchronize": ([P], ctypes.c_int),
             "swp_batch_destroy": ([P], ctypes.c_int),
             "swp_batch_kernel_launches": ([P], i64),
+            "swp_debug_batch_form": ([P, ctypes.POINTER(i64), ctypes.POINTER(i64)], ctypes.c_int),
             "swp_autotune_width": ([ctypes.POINTER(Desc), vp, i32, i64, ctypes.POINTER(i32)], ctypes.c_int),
             "swp_tuned_width": ([ctypes.POINTER(Desc), ctypes.POINTER(i32)], ctypes.c_int),
             "swp_autotune": ([ctypes.POINTER(Desc), vp, i32, i64, ctypes.POINTER(i32), ctypes.POINTER(i32)],
@@ -358,7 +359,8 @@ class Batch:
 
     def advance_ex(self, problems, steps, schemes=None, n=None, threads: int = 0, launch: str = "auto"):
         """Per-problem scheme ("swept", "classic" or "auto"; None = all auto)
-        and width (node or chunk); launch "auto" or "graph"."""
+        and width (node or chunk); launch "auto", "graph", or "persistent" (the
+        table form, where the given widths hold)."""
         count = len(problems)
         hs = (ctypes.c_void_p * count)(*[p._h.value for p in problems])
         st = _per_problem("steps", steps, count, ctypes.c_int64)
@@ -369,9 +371,9 @@ class Batch:
 
     def tune_width(self, problems, steps, candidates=(256, 512, 1024, 2048), threads: int = 0):
         """swp_batch_tune_width: each candidate target width fitted to every
-        problem's N and timed on one advance of the whole batch (states put
-        back after each); returns (widths of the fastest, its index, the
-        milliseconds of every candidate)."""
+        problem's N and timed on one "persistent" advance of the whole batch
+        (states put back after each); returns (widths of the fastest, its index,
+        the milliseconds of every candidate)."""
         count, nc = len(problems), len(candidates)
         hs = (ctypes.c_void_p * count)(*[p._h.value for p in problems])
         st = _per_problem("steps", steps, count, ctypes.c_int64)
@@ -388,6 +390,12 @@ class Batch:
 
     def kernel_launches(self) -> int:
         return int(self._lib.swp_batch_kernel_launches(self._h))
+
+    def debug_form(self):
+        """(problems that ran on chip, nodes and chunks of the table form) of the last advance."""
+        on_chip, nodes = ctypes.c_int64(0), ctypes.c_int64(0)
+        _check(self._lib.swp_debug_batch_form(self._h, ctypes.byref(on_chip), ctypes.byref(nodes)), "debug_batch_form")
+        return on_chip.value, nodes.value
 
     def close(self):
         if self._h and self._h.value:
