@@ -62,9 +62,9 @@ typedef enum { SWP_BC_PERIODIC = 0, SWP_BC_REFLECTIVE = 1, SWP_BC_DIRICHLET = 2 
 typedef enum { SWP_F64 = 0, SWP_F32 = 1 } swp_dtype;   /* Euler: SWP_F64 only */
 
 /* SWP_SCHEME_AUTO: the scheme (and width) swp_autotune measured faster for
- * the problem's (equation, dtype, n_points); swept at the tuned or default
- * width when none was measured; classic when N is too small for any swept
- * node width. */
+ * the problem's (equation, dtype, n_points); swept with the default launch and
+ * width when none was measured or when those measured faster still; classic when
+ * N is too small for any swept node width. */
 typedef enum { SWP_CLASSIC = 0, SWP_SWEPT = 1, SWP_SCHEME_AUTO = 2 } swp_scheme;
 
 /* Problem description.
@@ -174,7 +174,7 @@ swp_status swp_write(swp_problem* p, const void* src, size_t src_bytes, int src_
  * the N = K n + d points form K = floor(N / n) nodes, node k starting at
  * k n + floor(k d / K), so some are wider (by at most ceil(d / K) points);
  * such a split needs K >= 2.
- * 0 picks a width (the tuned one, else a default); when N is too small for
+ * 0 picks a width (see SWP_LAUNCH_AUTO); when N is too small for
  * any (fewer than two nodes of 4 * radius points) the advance runs the
  * classic scheme, whose result is the same.  The advance ends on a closing triangle, so
  * the state is complete afterwards (Section 4.2: output only at closing
@@ -256,9 +256,10 @@ swp_status swp_batch_create(void* cuda_stream, swp_batch** out);
 /* Advance problems[i] by n_steps[i] timesteps (swept), i < count.
  * points_per_block: per-problem node widths (any width swp_advance accepts),
  * or NULL / 0 entries for the tuned width of swp_autotune_width (else the
- * default rule, for Euler one that goes by the batch's cells; a problem too small for any node width runs as classic
- * items, with the same result).  threads: block
- * size (0 = 128 for FP64 and 32 for FP32; Euler at most 256).  Problems must be distinct.  Asynchronous;
+ * default rule, for Euler one that goes by the batch's cells; a problem too small
+ * for any node width runs as classic items, with the same result).  threads: block
+ * size (0 = 128 for FP64 and 32 for FP32; Euler at most 256).  Problems must be
+ * distinct.  Asynchronous;
  * SWP_ETIMEOUT surfaces at swp_batch_synchronize (wait bound as for
  * swp_advance's persistent launch, SWP_WAIT_LIMIT_NS included). */
 swp_status swp_batch_advance(swp_batch* b, swp_problem* const* problems, const int64_t* n_steps,
@@ -291,8 +292,13 @@ int64_t swp_batch_kernel_launches(const swp_batch* b);
 /* Node-width autotuner.  Times batch_count copies of the problem (initial
  * state u0_host, host memory) advanced `steps` timesteps in one batch for
  * every power-of-two node width up to 1024 that fits, keeps the fastest for the
- * (equation, dtype, n_points) of desc, and returns it in best_n.  Later
- * batches use it for problems of that key.  Allocates and frees its own
+ * (equation, dtype, n_points) of desc, and returns it in best_n.  The default
+ * launch of the same batch (the on-chip form, or the table form with the library's
+ * widths) is timed beside them: later batches use best_n for problems of that key
+ * where it was the faster one, or where the table form runs without a default rule of
+ * its own (beside classic problems, FP32 groups too long for the chip, the server's
+ * rounds).  A single default advance is timed against best_n too, and later single
+ * SWP_SCHEME_AUTO advances take the faster.  Allocates and frees its own
  * trial problems; synchronises the device. */
 swp_status swp_autotune_width(const swp_desc* desc, const void* u0_host, int32_t batch_count,
                               int64_t steps, int32_t* best_n);
@@ -302,10 +308,11 @@ swp_status swp_tuned_width(const swp_desc* desc, int32_t* n);
 /* Scheme autotuner.  Times the swept widths as swp_autotune_width does and
  * the classic scheme in the same batched form (chunks of 256, 1024 and 4096
  * points, capped at N), keeps whichever is faster for desc's (equation,
- * dtype, n_points) and returns it: best_scheme SWP_SWEPT or SWP_CLASSIC,
- * best_n its node or chunk width.  SWP_SCHEME_AUTO advances (single or
- * batched) of problems with that key then use it.  Allocates and frees its
- * own trial problems; synchronises the device. */
+ * dtype, n_points) and returns it: best_scheme SWP_SWEPT (the widths or the default
+ * launch won) or SWP_CLASSIC, best_n its node or chunk width.  SWP_SCHEME_AUTO
+ * advances of problems with that key then use it, batched ones as
+ * swp_autotune_width says, single ones unless the default launch was faster alone.
+ * Allocates and frees its own trial problems; synchronises the device. */
 swp_status swp_autotune(const swp_desc* desc, const void* u0_host, int32_t batch_count, int64_t steps,
                         int32_t* best_scheme, int32_t* best_n);
 /* The tuned choice for desc's key: scheme and width (SWP_SWEPT, 0 if none). */

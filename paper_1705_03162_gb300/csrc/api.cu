@@ -235,6 +235,8 @@ struct Tuned {
     int scheme = SWP_SWEPT;   // the faster scheme (swp_autotune)
     int n = 0;                // its width: swept node or classic chunk
     int n_swept = 0;          // the fastest swept node width
+    bool width_won = false;   // it beat the default launch (form and widths) in a batch
+    bool single_default = false;   // a single default swept advance beat the choice above
 };
 std::mutex g_tune_mutex;
 std::map<std::tuple<int, int, int64_t>, Tuned> g_tuned;
@@ -266,7 +268,7 @@ int width_for(const swp_problem* p, bool dataflow = false)
 int euler_batch_width(const swp_problem* p, int64_t cells)
 {
     Tuned t;
-    if (tuned_of(p->desc, &t) && t.n_swept > 0 && check_width(p, t.n_swept) == SWP_OK) return t.n_swept;
+    if (tuned_of(p->desc, &t) && t.width_won && check_width(p, t.n_swept) == SWP_OK) return t.n_swept;
     // (a short problem among large ones keeps some 48 nodes: its own chain of
     // phases would outlast the rest)
     const int64_t target =
@@ -692,9 +694,12 @@ swp_status advance_typed(swp_problem* p, int64_t steps, const swp_advance_opts& 
     if (o.scheme == SWP_SCHEME_AUTO) {
         int n = 0;
         choice_for(p, &o.scheme, &n);
-        // a measured width; without one the default launch and width
+        // a measured width; without one, or where it lost, the default launch and width
         Tuned t;
-        if (o.scheme == SWP_SWEPT && o.points_per_block == 0 && tuned_of(p->desc, &t) && t.n_swept > 0)
+        const bool tuned = tuned_of(p->desc, &t);
+        if (tuned && t.single_default && o.points_per_block == 0 && o.launch == SWP_LAUNCH_AUTO && o.threads == 0)
+            o.scheme = SWP_SWEPT;
+        else if (o.scheme == SWP_SWEPT && o.points_per_block == 0 && tuned && t.n_swept > 0)
             o.points_per_block = n;
     }
     if (o.scheme == SWP_SWEPT && o.points_per_block == 0 && o.launch != SWP_LAUNCH_REGISTER &&
@@ -1291,6 +1296,12 @@ bool resident_batch_group(swp_batch* b, std::vector<BatchItem>& plans, bool tabl
     if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, b->device) != cudaSuccess || !coop) return false;
     for (const auto& it : plans)
         if (it.kind != BATCH_SWEPT || it.s.T >= ((int64_t)1 << 31)) return false;
+    // a width measured faster than the default launch stays, unless another was given
+    auto won = [](const BatchItem& it) {
+        Tuned t;
+        return tuned_of(it.p->desc, &t) && t.width_won && t.n_swept == it.s.n;
+    };
+    if (std::all_of(plans.begin(), plans.end(), won)) return false;
     std::vector<int64_t> points;
     for (const auto& it : plans) points.push_back(it.p->N);
     ResidentBatchShape shape;
@@ -1304,9 +1315,7 @@ bool resident_batch_group(swp_batch* b, std::vector<BatchItem>& plans, bool tabl
         if (longest > kLongProblem) return false;
         const int64_t target = batch_width(total);
         for (auto& it : plans) {
-            if (table && it.given) continue;
-            Tuned t;   // (a width tuned for the problem, and not overridden, stays)
-            if (tuned_of(it.p->desc, &t) && t.n_swept == it.s.n) continue;
+            if ((table && it.given) || won(it)) continue;
             const int n = (int)fitted_width(it.p->rad, it.p->N, target);
             if (n == 0 || n == it.s.n || check_width(it.p, n) != SWP_OK) continue;
             it.s = plan_swept(it.p, it.s.T / it.p->sub, n);
@@ -1623,9 +1632,65 @@ done:
     return rate;
 }
 
-// Fastest swept node width (powers of two that fit) for the description.
+// Point-updates per second of one problem's advance (SWP_LAUNCH_AUTO) with the given
+// scheme and width (0: the default launch), or < 0.  Two untimed advances (a cached
+// graph is captured per starting row), then two timed.
+double time_single(const swp_desc* desc, const void* u0, int64_t steps, int scheme, int n)
+{
+    swp_problem* p = nullptr;
+    if (swp_create(desc, u0, 0, nullptr, &p) != SWP_OK) return -1.0;
+    double rate = -1.0;
+    cudaEvent_t e0 = nullptr, e1 = nullptr;
+    bool ok = cudaEventCreate(&e0) == cudaSuccess && cudaEventCreate(&e1) == cudaSuccess;
+    const int width = scheme == SWP_SWEPT ? n : 0;
+    for (int rep = 0; rep < 4 && ok; ++rep) {
+        if (rep == 2) ok = swp_synchronize(p) == SWP_OK && cudaEventRecord(e0, nullptr) == cudaSuccess;
+        ok = ok && swp_advance(p, steps, scheme, width) == SWP_OK;
+    }
+    float ms = 0.f;
+    if (ok && cudaEventRecord(e1, nullptr) == cudaSuccess && swp_synchronize(p) == SWP_OK &&
+        cudaEventElapsedTime(&ms, e0, e1) == cudaSuccess && ms > 0.f)
+        rate = 2.0 * (double)desc->n_points * (double)steps / (ms * 1e-3);
+    if (e0) cudaEventDestroy(e0);
+    if (e1) cudaEventDestroy(e1);
+    swp_destroy(p);
+    return rate;
+}
+
+// While it lives nothing is tuned for this key, so that default launches can be timed;
+// afterwards what was tuned before, or what keep() was given, is.
+struct TuneKey {
+    std::tuple<int, int, int64_t> key;
+    bool had = false;
+    Tuned t;
+    explicit TuneKey(const swp_desc* d) : key(d->eq, d->dtype, d->n_points)
+    {
+        std::lock_guard<std::mutex> lock(g_tune_mutex);
+        auto it = g_tuned.find(key);
+        if (it == g_tuned.end()) return;
+        had = true;
+        t = it->second;
+        g_tuned.erase(it);
+    }
+    void keep(const Tuned& now)
+    {
+        t = now;
+        had = true;
+    }
+    ~TuneKey()
+    {
+        if (!had) return;
+        std::lock_guard<std::mutex> lock(g_tune_mutex);
+        g_tuned[key] = t;
+    }
+    TuneKey(const TuneKey&) = delete;
+    TuneKey& operator=(const TuneKey&) = delete;
+};
+
+// Fastest swept node width (powers of two that fit) for the description, and the rate of
+// the default launch (form and widths chosen by the library) of the same batch.
 swp_status tune_swept(const swp_desc* desc, const void* u0_host, int32_t count, int64_t steps, int* best_n,
-                      double* best_rate)
+                      double* best_rate, double* default_rate)
 {
     swp_problem probe;   // for the width checks only
     probe.desc = *desc;
@@ -1649,6 +1714,7 @@ swp_status tune_swept(const swp_desc* desc, const void* u0_host, int32_t count, 
         }
     }
     if (*best_n == 0) return fail(SWP_EINVAL, "no node width could be timed for n_points %lld", (long long)probe.N);
+    *default_rate = time_batch(desc, u0_host, count, steps, SWP_SWEPT, 0, 0);
     return SWP_OK;
 }
 
@@ -1814,13 +1880,16 @@ swp_status swp_autotune_width(const swp_desc* desc, const void* u0_host, int32_t
         return fail(SWP_EINVAL, "u0_host / best_n NULL or count, steps <= 0");
     *best_n = 0;
     int n = 0;
-    double rate = 0.0;
-    if ((st = tune_swept(desc, u0_host, batch_count, steps, &n, &rate)) != SWP_OK) return st;
+    double rate = 0.0, default_rate = 0.0;
+    TuneKey key(desc);
+    if ((st = tune_swept(desc, u0_host, batch_count, steps, &n, &rate, &default_rate)) != SWP_OK) return st;
     *best_n = n;
-    std::lock_guard<std::mutex> lock(g_tune_mutex);
-    Tuned& t = g_tuned[std::make_tuple(desc->eq, desc->dtype, desc->n_points)];
+    Tuned t = key.t;   // (an earlier choice of the scheme stays)
     t.n_swept = n;
+    t.width_won = rate > default_rate;
     if (t.scheme == SWP_SWEPT) t.n = n;
+    t.single_default = time_single(desc, u0_host, steps, SWP_SWEPT, 0) >= time_single(desc, u0_host, steps, t.scheme, t.n);
+    key.keep(t);
     return SWP_OK;
 }
 
@@ -1834,8 +1903,9 @@ swp_status swp_autotune(const swp_desc* desc, const void* u0_host, int32_t batch
     *best_scheme = SWP_SWEPT;
     *best_n = 0;
     int n = 0;
-    double swept_rate = 0.0;
-    if ((st = tune_swept(desc, u0_host, batch_count, steps, &n, &swept_rate)) != SWP_OK) return st;
+    double swept_rate = 0.0, default_rate = 0.0;
+    TuneKey key(desc);
+    if ((st = tune_swept(desc, u0_host, batch_count, steps, &n, &swept_rate, &default_rate)) != SWP_OK) return st;
     // classic in the same batched form: chunks of 256 .. 4096 points
     int cm = 0;
     double classic_rate = -1.0;
@@ -1855,16 +1925,18 @@ swp_status swp_autotune(const swp_desc* desc, const void* u0_host, int32_t batch
         }
         if (mm == desc->n_points) break;
     }
-    std::lock_guard<std::mutex> lock(g_tune_mutex);
-    Tuned& t = g_tuned[std::make_tuple(desc->eq, desc->dtype, desc->n_points)];
+    Tuned t;
     t.n_swept = n;
-    if (cm > 0 && classic_rate > swept_rate) {
+    t.width_won = swept_rate > default_rate;
+    if (cm > 0 && classic_rate > std::max(swept_rate, default_rate)) {
         t.scheme = SWP_CLASSIC;
         t.n = cm;
     } else {
         t.scheme = SWP_SWEPT;
         t.n = n;
     }
+    t.single_default = time_single(desc, u0_host, steps, SWP_SWEPT, 0) >= time_single(desc, u0_host, steps, t.scheme, t.n);
+    key.keep(t);
     *best_scheme = t.scheme;
     *best_n = t.n;
     return SWP_OK;
