@@ -240,7 +240,8 @@ size_t swp_memory_in_use(void);
  * are checked and otherwise unused; they hold with SWP_LAUNCH_PERSISTENT (always the
  * table form) and with a given block size.  A problem above about 1,100,000 points
  * (FP32) or 900,000 (FP64, in a group too large for the on-chip form) sends the group
- * to the table form with the given widths.
+ * to the table form with the given widths, and so does a device that cannot hold the
+ * on-chip launch's blocks at once or its words in memory.
  * Each problem's result is bit-identical to swp_advance with the same scheme
  * (and, swept, the same node width).  The table costs 12 bytes of device
  * memory per (problem, phase) task, the on-chip form's halo words at most about
@@ -419,6 +420,10 @@ swp_status swp_debug_withhold_flags(swp_problem* p, int withhold, int64_t wait_l
 /* For tests: what form the batch's last advance took.  *on_chip: problems that ran
  * in the on-chip form; *nodes: nodes (classic: chunks) of those in the table form. */
 swp_status swp_debug_batch_form(const swp_batch* b, int64_t* on_chip, int64_t* nodes);
+/* For tests: refuse != 0 makes the batch's later on-chip launches fail on the host as
+ * if the device could not hold all their blocks at once (cudaErrorCooperativeLaunchTooLarge),
+ * for which the batch takes the table form; 0 restores it. */
+swp_status swp_debug_batch_refuse(swp_batch* b, int refuse);
 
 /* Swept advance that allocates nothing.  The paper has no counterpart: it is
  * here for callers that cannot call cudaMalloc -- code whose device memory is

@@ -1057,6 +1057,8 @@ struct swp_batch {
     cudaStream_t capture_stream = nullptr;
     uint64_t wait_limit_ns = 2000000000ull;
     int64_t on_chip = 0, nodes = 0;    // of the last advance: problems on chip, nodes and chunks of the table form
+    bool no_on_chip = false;           // the device cannot hold the on-chip launch's blocks at once
+    bool refuse_on_chip = false;       // test hook: its launches fail so
 };
 
 namespace {
@@ -1157,18 +1159,30 @@ bool batch_replay(swp_batch* b, const std::vector<int64_t>& key, swp_status* st)
 
 // Upload a launch's tables and run it: zero nctr counters and nflags flag words,
 // then launch(tables, stream), on the batch's stream or captured as a graph
-// with tables of its own under `key`.
+// with tables of its own under `key`.  refused, where given: set (and nothing
+// launched) when the tables do not fit in device memory, or, with
+// b->no_on_chip, when the device cannot hold a cooperative launch's blocks.
 template <typename Launch>
 swp_status batch_launch(swp_batch* b, const std::vector<BatchItem>& items, std::vector<int64_t> key, const void* insts,
                         size_t inst_bytes, const std::vector<int2>& tasks, size_t nctr, size_t nflags, bool graph,
-                        Launch launch)
+                        Launch launch, bool* refused = nullptr)
 {
+    auto too_large = [&](cudaError_t e) {
+        if (!refused || e != cudaErrorCooperativeLaunchTooLarge) return false;
+        cudaGetLastError();
+        b->no_on_chip = *refused = true;
+        return true;
+    };
     BatchGraph gnew;
     BatchTables& t = graph ? gnew.t : b->t;
     const size_t task_bytes = sizeof(int2) * tasks.size();
     swp_status st = grow_tables(t, inst_bytes, tasks.size(), nctr, nflags);
     if (st != SWP_OK) {
         if (graph) gnew.t.release();
+        if (refused && st == SWP_ENOMEM) {
+            cudaGetLastError();
+            *refused = true;
+        }
         return st;
     }
     // upload through the pinned staging buffer once its previous upload is done
@@ -1201,7 +1215,7 @@ swp_status batch_launch(swp_batch* b, const std::vector<BatchItem>& items, std::
     };
     if (!graph) {
         e = run(b->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "batch launch");
+        if (e != cudaSuccess) return too_large(e) ? SWP_ECUDA : cuda_fail(e, "batch launch");
     } else {
         // the uploads above are ordinary stream work; the graph holds the rest
         if (!b->capture_stream) {
@@ -1225,7 +1239,7 @@ swp_status batch_launch(swp_batch* b, const std::vector<BatchItem>& items, std::
             if (gnew.exec) cudaGraphExecDestroy(gnew.exec);
             cudaStreamSynchronize(b->stream);
             gnew.t.release();
-            return cuda_fail(e, "batch graph capture");
+            return too_large(e) ? SWP_ECUDA : cuda_fail(e, "batch graph capture");
         }
         gnew.key = std::move(key);
         for (const auto& it : items) {
@@ -1282,10 +1296,10 @@ constexpr int64_t kLongProblem = 900000;
 
 // The batched resident launch of whole heat / KS advances (resident_batch.cu).
 // False (nothing launched) when the dataflow launch takes them: a problem has more
-// tiles than the launch has blocks, the launch cannot run cooperatively, the stream is
-// being captured, or the dataflow launch is faster, for which the plans get widths by
-// the batch's size.  table: the caller asks for the dataflow launch, where the widths
-// that it gave hold.
+// tiles than the launch has blocks, the launch cannot run cooperatively or with the
+// device memory there is, the stream is being captured, or the dataflow launch is
+// faster, for which the plans get widths by the batch's size.  table: the caller asks
+// for the dataflow launch, where the widths that it gave hold.
 constexpr int kFormResident = 100;   // batch_key form, beside the dataflow modes
 
 template <typename R>
@@ -1323,7 +1337,7 @@ bool resident_batch_group(swp_batch* b, std::vector<BatchItem>& plans, bool tabl
             it.flip = (it.s.top & 1) != 0;
         }
     }
-    if (fit != RESIDENT_FITS || table) return false;
+    if (fit != RESIDENT_FITS || table || b->no_on_chip) return false;
     std::vector<BatchItem> items = plans;
     for (auto& it : items) it.flip = true;   // from one row to the other
     std::vector<int64_t> key;
@@ -1357,14 +1371,16 @@ bool resident_batch_group(swp_batch* b, std::vector<BatchItem>& plans, bool tabl
     w.ntiles = (int)tiles.size();
     w.status = b->status;
     w.wait_limit_ns = b->wait_limit_ns;
+    bool refused = false;
     *st = batch_launch(b, items, std::move(key), insts.data(), sizeof(ResidentInst<R>) * insts.size(), tiles, 1,
                        2 * (size_t)words, graph, [&](const BatchTables& t, cudaStream_t s) {
+                           if (b->refuse_on_chip) return cudaErrorCooperativeLaunchTooLarge;
                            w.tiles = t.tasks;
                            w.next_tile = t.ctr;
                            w.words = (uint64_t*)t.flags;
                            return launch_swept_resident_batch<R>((const ResidentInst<R>*)t.insts, w, shape, s);
-                       });
-    return true;
+                       }, &refused);
+    return !refused;
 }
 
 // One persistent launch of the items (one equation group and dtype).  status,
@@ -1862,6 +1878,14 @@ swp_status swp_batch_destroy(swp_batch* b)
 }
 
 int64_t swp_batch_kernel_launches(const swp_batch* b) { return b ? b->launches : -1; }
+
+swp_status swp_debug_batch_refuse(swp_batch* b, int refuse)
+{
+    if (!b) return fail(SWP_EINVAL, "batch is NULL");
+    b->refuse_on_chip = refuse != 0;
+    if (!refuse) b->no_on_chip = false;
+    return SWP_OK;
+}
 
 swp_status swp_debug_batch_form(const swp_batch* b, int64_t* on_chip, int64_t* nodes)
 {

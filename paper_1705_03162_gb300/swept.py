@@ -45,6 +45,7 @@ ABI_SYMBOLS = (
     "swp_batch_advance_ex", "swp_autotune", "swp_tuned", "swp_fit_width", "swp_batch_tune_width",
     "swp_server_create", "swp_server_submit", "swp_server_poll", "swp_server_wait",
     "swp_server_stats", "swp_server_destroy", "swp_debug_batch_form",
+    "swp_debug_batch_refuse",
 )
 
 
@@ -126,6 +127,7 @@ def load_library(path: str = LIB_PATH):
             "swp_batch_synchronize": ([P], ctypes.c_int),
             "swp_batch_destroy": ([P], ctypes.c_int),
             "swp_batch_kernel_launches": ([P], i64),
+            "swp_debug_batch_refuse": ([P, ctypes.c_int], ctypes.c_int),
             "swp_debug_batch_form": ([P, ctypes.POINTER(i64), ctypes.POINTER(i64)], ctypes.c_int),
             "swp_autotune_width": ([ctypes.POINTER(Desc), vp, i32, i64, ctypes.POINTER(i32)], ctypes.c_int),
             "swp_tuned_width": ([ctypes.POINTER(Desc), ctypes.POINTER(i32)], ctypes.c_int),
@@ -390,6 +392,9 @@ class Batch:
 
     def kernel_launches(self) -> int:
         return int(self._lib.swp_batch_kernel_launches(self._h))
+
+    def debug_refuse(self, refuse: bool):
+        _check(self._lib.swp_debug_batch_refuse(self._h, int(bool(refuse))), "debug_batch_refuse")
 
     def debug_form(self):
         """(problems that ran on chip, nodes and chunks of the table form) of the last advance."""

@@ -79,3 +79,23 @@ def test_tune_width_times_the_widths_it_returns(dtype):
         assert b.debug_form() == (3, 0)
         b.synchronize()
     s.check(2)
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("launch", ["auto", "graph"])
+def test_refused_on_chip_launch_takes_the_table_form(dtype, launch):
+    """A device that cannot hold the cooperative launch: the same advance in the
+    table form, also later without asking again, and on chip once it can."""
+    s = Set(dtype, [1031, 2503, 4099], 100)
+    with S.Batch(s.stream) as b:
+        b.debug_refuse(True)
+        for _ in range(2):
+            b.advance_ex(s.probs, s.steps, ["swept"] * 3, launch=launch)
+            on_chip, nodes = b.debug_form()
+            assert on_chip == 0 and nodes >= 6
+        b.debug_refuse(False)
+        b.advance_ex(s.probs, s.steps, ["swept"] * 3, launch=launch)
+        assert b.debug_form() == (3, 0)
+        b.synchronize()
+        assert b.kernel_launches() == 3
+    s.check(3)
