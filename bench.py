@@ -95,7 +95,7 @@ NCU_TRAFFIC = {
 # instances of the batched workload; the on-chip tiles of resident_batch.cu): warp
 # instructions issued over 4 per SM per cycle, keyed like the traffic record
 # and reported when the timed batch runs on chip.
-NCU_ISSUE_FP32_BATCH = {"src": "b90796f1a92fd58a", "form": "on chip", "issue_frac": 0.715, "issue_active": 0.715,
+NCU_ISSUE_FP32_BATCH = {"src": "c8896dc45938305d", "form": "on chip", "issue_frac": 0.715, "issue_active": 0.715,
                         "fma_pipe": 0.635}
 KERNEL_OF_LAUNCH = {"per_phase": "swept_phase_kernel", "graph": "swept_phase_kernel",
                     "persistent": "swept_batch_kernel", "auto": "swept_batch_kernel"}

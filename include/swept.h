@@ -407,10 +407,12 @@ swp_status swp_server_destroy(swp_server* s);
 
 /* Fault-injection hook for tests of the bounded waits of persistent and on-chip
  * launches.  withhold != 0 makes every neighbour wait of later
- * SWP_LAUNCH_PERSISTENT and on-chip advances of this problem wait for a flag value no node ever publishes, so
- * each wait gives up after wait_limit_ns nanoseconds (device global timer),
- * the kernel returns without computing, and the next swp_synchronize /
- * swp_read reports SWP_ETIMEOUT (the state is then invalid).  withhold = 0
+ * SWP_LAUNCH_PERSISTENT and on-chip advances of this problem, and of a batch's
+ * on-chip launch with this problem in it, wait for a flag value no node ever
+ * publishes, so each wait gives up after wait_limit_ns nanoseconds (device global
+ * timer), the kernel returns without computing, and the next swp_synchronize /
+ * swp_read, or swp_batch_synchronize, reports SWP_ETIMEOUT (the state, or all of the
+ * launch's states, are then invalid).  withhold = 0
  * restores normal waits; wait_limit_ns (in (0, 1e10]) bounds every wait of
  * those advances either way (default 2 s).  Nothing faults, traps
  * or hangs.  The paper has no counterpart: its nodes synchronise only at

@@ -1340,9 +1340,19 @@ bool resident_batch_group(swp_batch* b, std::vector<BatchItem>& plans, bool tabl
     if (fit != RESIDENT_FITS || table || b->no_on_chip) return false;
     std::vector<BatchItem> items = plans;
     for (auto& it : items) it.flip = true;   // from one row to the other
+    ResidentBatchWork w;
+    w.wait_offset = 0;
+    w.wait_limit_ns = b->wait_limit_ns;
+    for (const auto& it : items)   // test hook: every wait of the launch
+        if (it.p->inject_withheld_flags) {
+            w.wait_limit_ns = w.wait_offset ? std::min(w.wait_limit_ns, it.p->wait_limit_ns) : it.p->wait_limit_ns;
+            w.wait_offset = withheld_offset(it.p);
+        }
     std::vector<int64_t> key;
     if (graph) {
         key = batch_key(items, kFormResident, 0);
+        key.push_back(w.wait_offset);
+        key.push_back((int64_t)w.wait_limit_ns);
         if (batch_replay(b, key, st)) return true;
     }
     std::vector<std::pair<double, int>> order(items.size());   // longest advance first
@@ -1367,10 +1377,8 @@ bool resident_batch_group(swp_batch* b, std::vector<BatchItem>& plans, bool tabl
         for (int k = 0; k < in.g.K; ++k) tiles.push_back(make_int2(i, k));
         in.last_tile = (int)tiles.size() - 1;
     }
-    ResidentBatchWork w;
     w.ntiles = (int)tiles.size();
     w.status = b->status;
-    w.wait_limit_ns = b->wait_limit_ns;
     bool refused = false;
     *st = batch_launch(b, items, std::move(key), insts.data(), sizeof(ResidentInst<R>) * insts.size(), tiles, 1,
                        2 * (size_t)words, graph, [&](const BatchTables& t, cudaStream_t s) {

@@ -81,6 +81,7 @@ struct ResidentBatchWork {
     uint64_t* words;       // zeroed per launch
     int* status;
     uint64_t wait_limit_ns;
+    uint32_t wait_offset;  // 0; a test hook sets it so that no wait can succeed
 };
 struct ResidentBatchShape {
     int variant = 0;       // of the kernel's tiles

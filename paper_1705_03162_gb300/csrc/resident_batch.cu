@@ -59,7 +59,7 @@ __global__ void __launch_bounds__(T::THREADS, T::BLOCKS_PER_SM)
         ResidentGeom g = in.g;
         g.sync.words = w.words + in.word_off;
         g.sync.seq = 1;
-        g.sync.wait_offset = 0;
+        g.sync.wait_offset = w.wait_offset;
         g.sync.wait_limit_ns = w.wait_limit_ns;
         g.sync.status = w.status;
         g.sync.claimed = w.next_tile;

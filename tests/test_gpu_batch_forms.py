@@ -1,5 +1,7 @@
 """Which form a batch of heat and KS problems takes (on chip, or the table form with
 which node widths), and that each gives the classic scheme's bits."""
+import time
+
 import numpy as np
 import pytest
 
@@ -99,3 +101,35 @@ def test_refused_on_chip_launch_takes_the_table_form(dtype, launch):
         b.synchronize()
         assert b.kernel_launches() == 3
     s.check(3)
+
+
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+@pytest.mark.parametrize("launch", ["auto", "graph"])
+def test_withheld_words_of_a_batch_time_out_and_recover(dtype, launch):
+    """Problems of several tiles among which one has its words withheld: every
+    wait of the launch gives up within the limit (blocks whose tiles are still
+    unclaimed leave too), synchronize reports it, and the batch runs again once
+    the states are rewritten."""
+    sizes = [1031, 4099, 2503, 30, 3000] if dtype == "f64" else [15000] * 90 + [4099, 30]
+    s = Set(dtype, sizes, 100)
+    schemes = ["swept"] * len(sizes)
+    with S.Batch(s.stream) as b:
+        b.advance_ex(s.probs, s.steps, schemes, launch=launch)
+        assert b.debug_form() == (len(sizes), 0)
+        b.synchronize()
+        s.probs[1].debug_withhold_flags(True, wait_limit_ns=100_000_000)
+        for _ in range(2):
+            t0 = time.perf_counter()
+            b.advance_ex(s.probs, s.steps, schemes, launch=launch)
+            assert b.debug_form() == (len(sizes), 0)
+            with pytest.raises(S.SweptError) as e:
+                b.synchronize()
+            assert e.value.status == S.ETIMEOUT
+            assert time.perf_counter() - t0 < 5
+        s.probs[1].debug_withhold_flags(False)
+        for p, u in zip(s.probs, s.u0):
+            p.write(u)
+        for _ in range(2):
+            b.advance_ex(s.probs, s.steps, schemes, launch=launch)
+        b.synchronize()
+    s.check(2)
