@@ -89,7 +89,7 @@ def alu_roofline(updates: float, seconds: float, eq: str, dtype: str) -> dict:
 NCU_TRAFFIC = {
     # dram__bytes_read.sum + dram__bytes_write.sum of the whole 10^4-step solve in
     # one dataflow launch: a one-pass capture of the benchmark's own timed launch
-    "swept_batch_kernel<double,KS> n=1024 threads=256": {"src": "b90796f1a92fd58a", "bytes_per_launch": 11520000},
+    "swept_batch_kernel<double,KS> n=1024 threads=256": {"src": "c8896dc45938305d", "bytes_per_launch": 11630000},
 }
 # Issue-slot use of the batched FP32 launch from one ncu capture (the 4096
 # instances of the batched workload; the on-chip tiles of resident_batch.cu): warp
