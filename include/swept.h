@@ -419,9 +419,16 @@ swp_status swp_server_destroy(swp_server* s);
  * kernel boundaries (Section 3). */
 swp_status swp_debug_withhold_flags(swp_problem* p, int withhold, int64_t wait_limit_ns);
 
+/* For tests: the problem's next on-chip advance numbers its exchanges from `next` (at
+ * least the number it would use, below 2^31; it starts over at 1 rather than pass
+ * 2^31).  SWP_EINVAL before the first on-chip advance. */
+swp_status swp_debug_sequence(swp_problem* p, int64_t next);
+
 /* For tests: what form the batch's last advance took.  *on_chip: problems that ran
  * in the on-chip form; *nodes: nodes (classic: chunks) of those in the table form. */
 swp_status swp_debug_batch_form(const swp_batch* b, int64_t* on_chip, int64_t* nodes);
+/* Their tiles, -1 for NULL: a problem of N points has ceil(N / points per tile). */
+int64_t swp_debug_batch_tiles(const swp_batch* b);
 /* For tests: refuse != 0 makes the batch's later on-chip launches fail on the host as
  * if the device could not hold all their blocks at once (cudaErrorCooperativeLaunchTooLarge),
  * for which the batch takes the table form; 0 restores it. */

@@ -990,6 +990,16 @@ swp_status swp_debug_withhold_flags(swp_problem* p, int withhold, int64_t wait_l
     return SWP_OK;
 }
 
+swp_status swp_debug_sequence(swp_problem* p, int64_t next)
+{
+    if (!p) return fail(SWP_EINVAL, "problem is NULL");
+    if (!p->words) return fail(SWP_EINVAL, "no on-chip advance has run");
+    if (next < (int64_t)p->seq || next >= (int64_t)1 << 31)
+        return fail(SWP_EINVAL, "next must be in [%u, 2^31)", p->seq);
+    p->seq = (uint32_t)next;
+    return SWP_OK;
+}
+
 const char* swp_status_str(swp_status s)
 {
     switch (s) {
@@ -1056,7 +1066,8 @@ struct swp_batch {
     std::vector<BatchGraph> graphs;    // at most 8, oldest first
     cudaStream_t capture_stream = nullptr;
     uint64_t wait_limit_ns = 2000000000ull;
-    int64_t on_chip = 0, nodes = 0;    // of the last advance: problems on chip, nodes and chunks of the table form
+    int64_t on_chip = 0, tiles = 0, nodes = 0;   // of the last advance: problems on chip and their tiles, nodes and
+                                                 // chunks of the table form
     bool no_on_chip = false;           // the device cannot hold the on-chip launch's blocks at once
     bool refuse_on_chip = false;       // test hook: its launches fail so
 };
@@ -1339,7 +1350,13 @@ bool resident_batch_group(swp_batch* b, std::vector<BatchItem>& plans, bool tabl
     }
     if (fit != RESIDENT_FITS || table || b->no_on_chip) return false;
     std::vector<BatchItem> items = plans;
-    for (auto& it : items) it.flip = true;   // from one row to the other
+    int64_t ntiles = 0;
+    for (auto& it : items) {
+        it.flip = true;   // from one row to the other
+        ntiles += resident_batch_geom(it.p->desc.eq, (int)sizeof(R), it.p->desc.bc, it.p->N, it.s.T, shape).K;
+    }
+    if (ntiles >= (int64_t)1 << 30) return false;
+    b->tiles += ntiles;
     ResidentBatchWork w;
     w.wait_offset = 0;
     w.wait_limit_ns = b->wait_limit_ns;
@@ -1373,7 +1390,6 @@ bool resident_batch_group(swp_batch* b, std::vector<BatchItem>& plans, bool tabl
         in.word_off = words;
         in.c = coefs_of<R>(p);
         if (in.g.K > 1) words += 2 * in.g.parity_words;
-        if ((int64_t)tiles.size() + in.g.K >= (int64_t)1 << 30) return false;
         for (int k = 0; k < in.g.K; ++k) tiles.push_back(make_int2(i, k));
         in.last_tile = (int)tiles.size() - 1;
     }
@@ -1525,7 +1541,7 @@ swp_status persistent_via_batch(swp_problem* p, const SweptPlan& s, int threads)
 swp_status launch_groups(swp_batch* b, std::vector<BatchItem> (&groups)[2][2], int threads, bool graph, bool whole,
                          bool table)
 {
-    b->on_chip = b->nodes = 0;
+    b->on_chip = b->tiles = b->nodes = 0;
     for (int g = 0; g < 2; ++g)
         for (int dt = 0; dt < 2; ++dt) {
             if (groups[g][dt].empty()) continue;
@@ -1886,6 +1902,8 @@ swp_status swp_batch_destroy(swp_batch* b)
 }
 
 int64_t swp_batch_kernel_launches(const swp_batch* b) { return b ? b->launches : -1; }
+
+int64_t swp_debug_batch_tiles(const swp_batch* b) { return b ? b->tiles : -1; }
 
 swp_status swp_debug_batch_refuse(swp_batch* b, int refuse)
 {

@@ -45,7 +45,7 @@ ABI_SYMBOLS = (
     "swp_batch_advance_ex", "swp_autotune", "swp_tuned", "swp_fit_width", "swp_batch_tune_width",
     "swp_server_create", "swp_server_submit", "swp_server_poll", "swp_server_wait",
     "swp_server_stats", "swp_server_destroy", "swp_debug_batch_form",
-    "swp_debug_batch_refuse",
+    "swp_debug_batch_refuse", "swp_debug_batch_tiles", "swp_debug_sequence",
 )
 
 
@@ -127,6 +127,8 @@ def load_library(path: str = LIB_PATH):
             "swp_batch_synchronize": ([P], ctypes.c_int),
             "swp_batch_destroy": ([P], ctypes.c_int),
             "swp_batch_kernel_launches": ([P], i64),
+            "swp_debug_sequence": ([P, i64], ctypes.c_int),
+            "swp_debug_batch_tiles": ([P], i64),
             "swp_debug_batch_refuse": ([P, ctypes.c_int], ctypes.c_int),
             "swp_debug_batch_form": ([P, ctypes.POINTER(i64), ctypes.POINTER(i64)], ctypes.c_int),
             "swp_autotune_width": ([ctypes.POINTER(Desc), vp, i32, i64, ctypes.POINTER(i32)], ctypes.c_int),
@@ -270,6 +272,9 @@ class Problem:
         _check(self._lib.swp_debug_withhold_flags(self._h, int(bool(withhold)), int(wait_limit_ns)),
                "debug_withhold_flags")
 
+    def debug_sequence(self, next_: int):
+        _check(self._lib.swp_debug_sequence(self._h, int(next_)), "debug_sequence")
+
     def close(self):
         if self._h and self._h.value:
             _check(self._lib.swp_destroy(self._h), "destroy")
@@ -392,6 +397,10 @@ class Batch:
 
     def kernel_launches(self) -> int:
         return int(self._lib.swp_batch_kernel_launches(self._h))
+
+    def debug_tiles(self) -> int:
+        """On-chip tiles of the last advance."""
+        return int(self._lib.swp_debug_batch_tiles(self._h))
 
     def debug_refuse(self, refuse: bool):
         _check(self._lib.swp_debug_batch_refuse(self._h, int(bool(refuse))), "debug_batch_refuse")
