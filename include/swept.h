@@ -97,7 +97,8 @@ typedef enum {
                                    blocks) where that is the faster form: heat
                                    and KS in FP64 up to 2^17 points, beyond that
                                    heat up to about 10^6; Euler up to about
-                                   330000 cells; heat and KS in FP32 up to about
+                                   330000 cells (Dirichlet ends: 57000);
+                                   heat and KS in FP32 up to about
                                    2*10^6 points, and in tiles of the same
                                    kind, a launch per some ten levels, above.
                                    Otherwise (wider FP64 grids, a given width,

@@ -461,7 +461,7 @@ bool run_swept_resident(swp_problem* p, int64_t steps, swp_status* st)
     if (!p->shape_known) {
         p->shape_known = true;
         const bool fits = p->desc.eq == SWP_EULER
-                              ? resident_euler_plan(p->N, p->sms, &p->shape)
+                              ? resident_euler_plan(p->desc.bc, p->N, p->sms, &p->shape)
                               : resident_plan(p->desc.eq, p->esize, p->N, p->sms, &p->shape);
         if (!fits) p->shape.K = 0;
     }

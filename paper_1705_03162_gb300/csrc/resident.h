@@ -99,7 +99,7 @@ cudaError_t launch_swept_resident_batch(const ResidentInst<R>* insts, const Resi
 
 // The same for Euler (FP64): cells in shared memory, L levels per exchange, M = 1, P
 // = 1 where the interfaces' sides are tasks of their own, else 0; warps unused.
-bool resident_euler_plan(int64_t N, int sms, ResidentShape* out);
+bool resident_euler_plan(int bc, int64_t N, int sms, ResidentShape* out);
 size_t resident_euler_words(int64_t N, const ResidentShape& s);
 cudaError_t launch_swept_resident_euler(int bc, const double* A, double* B, int64_t N, int64_t levels,
                                         const ResidentShape& s, const ResidentSync& y, const Coefs<double>& c,

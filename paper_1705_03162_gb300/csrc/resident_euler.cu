@@ -18,7 +18,8 @@
 // against the dataflow launch, Sod / limited everywhere: N = 4096 8100 / 8200
 // (21200 / 22600 when this form came), 65536 22500 / 32700 (28000 / 48700), 200000
 // 54000 / 91000 (62200 / 115100).  Grids whose cells do not fit shared memory (N above about
-// 330000) keep that launch.
+// 330000), and Dirichlet ones above about 57000 cells (resident_euler_plan), keep that
+// launch.
 //
 // Dirichlet ends: the tile's slots beyond an end hold that end's ghost state in
 // both rows and are never updated (Appendix C's two ghost cells, and more of
@@ -207,13 +208,27 @@ int turns(int n) { return ((n + 31) / 32 + 3) / 4; }
 
 }  // namespace
 
-bool resident_euler_plan(int64_t N, int sms, ResidentShape* out)
+bool resident_euler_plan(int bc, int64_t N, int sms, ResidentShape* out)
 {
     *out = ResidentShape();
     if (N < 32 || sms < 1) return false;
     const int K = (int)std::min<int64_t>(sms, std::max<int64_t>(1, N / 8));
     if ((N + 1) * (K + 1) >= (int64_t)1 << 31) return false;
     const int own = (int)((N + K - 1) / K);
+    // The blocks keep the pace of the slowest one, a tile limited everywhere, while the
+    // dataflow launch's is the average of the grid.  Dirichlet ends are a tube whose
+    // waves hold a part of it: beyond three turns of rows per pass (own + the shortest
+    // halos; 57152 cells on 152 SMs) the dataflow launch is the faster form.  us per step
+    // over 100 to 800 steps of the Sod tube, on chip / dataflow, at t = 0.03 / 0.1 / 0.2:
+    //    55109   25.3 / 24.9   25.3 / 25.7    25.4 / 33.7
+    //    60001   31.0 / 25.9   31.0 / 26.4    31.1 / 35.1
+    //    77936   42.4 / 28.4   42.5 / 29.0    42.7 / 38.9
+    //   131072   56.5 / 38.2   57.2 / 39.1    57.3 / 53.5
+    //   300001  126.7 / 78.8  127.3 / 80.7   128.1 / 111
+    // (its first steps, when hardly a cell is limited, are faster on chip: 131072 cells
+    // 35.6 / 37.1 over 250 steps.)  Periodic flows are mostly limited everywhere (131072:
+    // 57.5 / 68.9) and stay on chip.
+    if (bc == DIRICHLET && turns(own + 8) > 3) return false;
     double best = 0.0;
     for (int split = 0; split < 2; ++split)
         for (int L = 2; L <= 48; L += 2) {

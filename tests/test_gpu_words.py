@@ -1,5 +1,5 @@
 """The published words of a single on-chip advance: sequence numbers that start over,
-and waits that run out, in every kernel that polls them."""
+waits that run out, in every kernel that polls them, and which Euler grids have them."""
 import time
 
 import numpy as np
@@ -67,3 +67,21 @@ def test_withheld_words_time_out_and_recover(eq, bc, N, dtype):
         p.write(u0)
         p.advance(2000, "swept")
         assert np.array_equal(p.read(), _classic(spec, u0, dtype, 2000))
+
+
+@pytest.mark.parametrize("bc,N,on_chip", [("dirichlet", 57001, True), ("dirichlet", 57301, False),
+                                          ("dirichlet", 131072, False), ("periodic", 131072, True)])
+def test_euler_form_by_boundary(bc, N, on_chip):
+    """A Dirichlet tube's default advance leaves the chip where the dataflow launch
+    becomes the faster form (a problem without on-chip words has no sequence)."""
+    spec, u0 = _case("euler", bc, N, "f64")
+    with S.Problem(spec, u0, "f64") as p:
+        p.advance(12, "swept")
+        if on_chip:
+            p.debug_sequence(1 << 20)
+        else:
+            with pytest.raises(S.SweptError) as e:
+                p.debug_sequence(1 << 20)
+            assert e.value.status == S.EINVAL
+        p.advance(5, "swept")
+        assert np.array_equal(p.read(), _classic(spec, u0, "f64", 17))
