@@ -89,13 +89,13 @@ def alu_roofline(updates: float, seconds: float, eq: str, dtype: str) -> dict:
 NCU_TRAFFIC = {
     # dram__bytes_read.sum + dram__bytes_write.sum of the whole 10^4-step solve in
     # one dataflow launch: a one-pass capture of the benchmark's own timed launch
-    "swept_batch_kernel<double,KS> n=1024 threads=256": {"src": "005a281318cd6aa5", "bytes_per_launch": 11770000},
+    "swept_batch_kernel<double,KS> n=1024 threads=256": {"src": "b688f34d523dfd21", "bytes_per_launch": 12070000},
 }
 # Issue-slot use of the batched FP32 launch from one ncu capture (the 4096
 # instances of the batched workload; the on-chip tiles of resident_batch.cu): warp
 # instructions issued over 4 per SM per cycle, keyed like the traffic record
 # and reported when the timed batch runs on chip.
-NCU_ISSUE_FP32_BATCH = {"src": "005a281318cd6aa5", "form": "on chip", "issue_frac": 0.715, "issue_active": 0.715,
+NCU_ISSUE_FP32_BATCH = {"src": "b688f34d523dfd21", "form": "on chip", "issue_frac": 0.715, "issue_active": 0.715,
                         "fma_pipe": 0.635}
 KERNEL_OF_LAUNCH = {"per_phase": "swept_phase_kernel", "graph": "swept_phase_kernel",
                     "persistent": "swept_batch_kernel", "auto": "swept_batch_kernel"}

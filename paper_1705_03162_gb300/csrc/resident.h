@@ -28,6 +28,7 @@ struct ResidentShape {
     int P = 0;        // points per thread
     int warps = 0;    // warps per block
     int L = 0, M = 0; // levels per warp round, rounds per exchange between blocks
+    bool split = false;   // Euler: the sides of an interface are tasks of their own
 };
 // What a launch synchronises through: two sets of published words (one per
 // exchange parity), each word carrying the exchange's sequence number, which
@@ -97,8 +98,8 @@ template <typename R>
 cudaError_t launch_swept_resident_batch(const ResidentInst<R>* insts, const ResidentBatchWork& w,
                                         const ResidentBatchShape& shape, cudaStream_t s);
 
-// The same for Euler (FP64): cells in shared memory, L levels per exchange, M = 1, P
-// = 1 where the interfaces' sides are tasks of their own, else 0; warps unused.
+// The same for Euler (FP64): cells in shared memory, L levels per exchange, M = 1; P and
+// warps unused.
 bool resident_euler_plan(int bc, int64_t N, int sms, ResidentShape* out);
 size_t resident_euler_words(int64_t N, const ResidentShape& s);
 cudaError_t launch_swept_resident_euler(int bc, const double* A, double* B, int64_t N, int64_t levels,

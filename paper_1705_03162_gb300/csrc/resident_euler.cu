@@ -240,7 +240,8 @@ bool resident_euler_plan(int bc, int64_t N, int sms, ResidentShape* out)
             for (int j = 1; j <= L; ++j) {
                 const int n = W - 4 * j;
                 const int flux = split ? 28 * turns(2 * n + 2) + 33 * turns(n + 1) : 82 * turns(n + 1);
-                const int cell = split ? 10 * turns(2 * ((n + 4 + 31) & ~31)) + 12 * turns(n + 2) : 11 * turns(n + 4) + 20 * turns(n + 2);
+                const int cell = split ? 10 * turns(2 * ((n + 4 + 31) & ~31)) + 12 * turns(n + 2)
+                                       : 11 * turns(n + 4) + 20 * turns(n + 2);
                 clocks += 66.0 * (cell + flux + 6 * turns(n)) + (split ? 700.0 : 500.0);
             }
             clocks /= L;
@@ -249,7 +250,7 @@ bool resident_euler_plan(int bc, int64_t N, int sms, ResidentShape* out)
                 out->K = K;
                 out->L = L;
                 out->M = 1;
-                out->P = split;
+                out->split = split != 0;
             }
         }
     return best > 0.0;
@@ -278,12 +279,13 @@ cudaError_t launch_swept_resident_euler(int bc, const double* A, double* B, int6
     g.bc = bc;
     g.sync = y;
     g.parity_words = (int64_t)resident_euler_words(N, s);
-    const size_t smem = smem_of(own, s.L, s.P != 0);
-    const void* fn = s.P ? (const void*)swept_resident_euler_kernel<true> : (const void*)swept_resident_euler_kernel<false>;
+    const size_t smem = smem_of(own, s.L, s.split);
+    const void* fn = s.split ? (const void*)swept_resident_euler_kernel<true>
+                             : (const void*)swept_resident_euler_kernel<false>;
     const cudaError_t e = allow_resident_smem(fn);
     if (e != cudaSuccess) return e;
     void* args[] = {(void*)&A, (void*)&B, (void*)&g, (void*)&c};
-    return cudaLaunchCooperativeKernel(fn, dim3((unsigned)s.K), dim3(s.P ? kThreads<true> : kThreads<false>), args,
+    return cudaLaunchCooperativeKernel(fn, dim3((unsigned)s.K), dim3(s.split ? kThreads<true> : kThreads<false>), args,
                                        smem, st);
 }
 
