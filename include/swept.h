@@ -101,8 +101,9 @@ typedef enum {
                                    heat and KS in FP32 up to about
                                    2*10^6 points, and in tiles of the same
                                    kind, a launch per some ten levels, above.
-                                   Otherwise (wider FP64 grids, a given width,
-                                   a stream under capture): periodic heat
+                                   Otherwise (wider FP64 grids, a stream under
+                                   capture, a device that cannot hold that
+                                   launch or its words): periodic heat
                                    and KS with N a multiple of 32, CLUSTER up to
                                    N = 2048 (FP64) or 4096 (FP32), then
                                    REGISTER up to 2^15 for FP64 heat, 2^14
@@ -110,7 +111,9 @@ typedef enum {
                                    FP32 KS;
                                    otherwise in FP64 GRAPH
                                    below 2^17 and PERSISTENT from 2^17
-                                   (Euler: from 2^13), in FP32 PER_PHASE */
+                                   (Euler: from 2^13), in FP32 PER_PHASE.
+                                   A given width or block size goes straight
+                                   to these three */
     SWP_LAUNCH_PER_PHASE = 1,   /* one kernel per triangle / diamond phase;
                                    nodes synchronise at kernel boundaries */
     SWP_LAUNCH_PERSISTENT = 2,  /* one dataflow kernel for the whole advance
@@ -245,8 +248,9 @@ size_t swp_memory_in_use(void);
  * on-chip launch's blocks at once or its words in memory.
  * Each problem's result is bit-identical to swp_advance with the same scheme
  * (and, swept, the same node width).  The table costs 12 bytes of device
- * memory per (problem, phase) task, the on-chip form's halo words at most about
- * 2 KB per 1000 points; this workspace is not counted against
+ * memory per (problem, phase) task; the on-chip form's halo words take about 2 KB
+ * per 1000 points in FP32 and 12.5 KB in FP64 (at most twice that, for a problem of
+ * just more than one tile).  This workspace is not counted against
  * swp_set_memory_budget.  A batch, like its problems, is used by one host
  * thread at a time.  The paper has no batched form. */
 typedef struct swp_batch swp_batch;
@@ -339,7 +343,8 @@ swp_status swp_fit_width(int32_t eq, int64_t n_points, int32_t target, int32_t* 
  * stream (the span includes the host building and uploading the task tables, as a
  * plain advance would).  Run the chosen widths with SWP_LAUNCH_PERSISTENT or the same
  * given block size: SWP_LAUNCH_AUTO and _GRAPH with the default block size choose form
- * and widths themselves, mostly the faster way.  A problem listed twice is rejected by the advance
+ * and widths themselves, mostly the faster way.  A problem listed twice is rejected
+ * by the advance
  * (SWP_EINVAL) after the states are saved, and put back.  The
  * fastest candidate's per-problem widths are written to widths_out[count],
  * its index to *best (may be NULL), and each candidate's milliseconds to
