@@ -20,7 +20,8 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libswept.so")
-SOURCES = ["api.cu", "classic.cu", "swept.cu", "register.cu", "resident.cu", "resident_batch.cu", "resident_euler.cu", "server.cu"]
+SOURCES = ["api.cu", "classic.cu", "swept.cu", "register.cu", "resident.cu", "resident_batch.cu",
+           "resident_euler.cu", "server.cu"]
 HEADERS = ["scheme.cuh", "launch.h", "geometry.cuh", "resident.h", "resident.cuh", "resident_tile.cuh"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 

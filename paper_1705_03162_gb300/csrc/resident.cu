@@ -36,17 +36,23 @@
 // Each point update is scheme.cuh's on the same operands as in the classic
 // scheme, so the bits are the same.
 //
-// What bounds it.  FP64: its pipe, at 66 clocks per warp-wide FMA; with one warp
-// per SM sub-partition the chain of a level (KS N = 1024: 550 of 670 clocks),
-// and the exchange of about 1450 clocks between blocks.  FP32: instruction
-// issue; 94 % of the instructions are the point updates' own, and the slots that
-// eligible warps leave unused are lost to their register operands (Pair).  Measured per advance against the forms that were the
-// default before (cluster, Register and Shared graphs, per-phase FP32):
-//   heat FP64 N = 1024, 4096 steps      1196 -> 610 us
-//   heat FP64 reflective 50001, 2000    1559 -> 807 us
-//   KS FP64 10007, 2000 steps           3224 -> 1492 us
-//   heat FP32 2^17, 4000 steps          1080 -> 178 us
-//   KS FP32 2000003, 1000 steps         3710 -> 1021 us
+// What bounds it.  FP64: its pipe, a warp-wide FMA every 64 clocks; with one warp
+// per SM sub-partition the chain of a level (KS N = 1024: 569 of 667 clocks per level)
+// and the exchange between blocks (1340 to 1530 clocks each, clock counters of all
+// blocks).  FP32 KS: the FMA pipe, 80 % of it in pairs (an f32x2 takes it two clocks;
+// "math pipe throttle" is the top stall).  FP32 heat at 2^17: one warp per
+// sub-partition, 59 clocks a level of which 41 % issue, and exchanges of 2940 clocks
+// (192 halo points a side) every 192 levels.  86 % of the FP32 instructions are the
+// point updates' own.  Measured per advance (write, advance, read) against the forms
+// that were the default before (cluster, Register and Shared graphs, per-phase FP32):
+//   heat FP64 N = 1024, 4096 steps      1193 -> 615 us
+//   heat FP64 reflective 50001, 2000    1556 -> 806 us
+//   KS FP64 10007, 2000 steps           3217 -> 1537 us
+//   heat FP32 2^17, 4000 steps          1078 -> 178 us
+//   KS FP32 2000003, 1000 steps         3699 -> 1024 us
+// and beyond the chip, a launch per exchange, in G point-updates/s: heat FP32 2^22
+// 1585 -> 6950, 2^24 1640 -> 6490, 2^26 1430 -> 3650; KS FP32 2^22 583 -> 1619, 2^24
+// 589 -> 1456, 2^26 575 -> 1257.
 #include <algorithm>
 
 #include "resident.h"
@@ -121,14 +127,17 @@ constexpr int kPoints32[] = {1, 2, 4, 8, 12, 16, 20, 24, 28, 32};
 
 namespace {
 
-// Estimated clocks (2.07 GHz) per level of a block of `warps` warps with P
-// points per thread that owns its tile's points, from a fit to 2294 measured
-// shapes (N from 2^10 to 2^21): the arithmetic of a level, the round through
-// shared memory every L levels (170 to 1000) and the exchange between blocks
-// every L M levels (1450 and the polls of its halo).  FP64 is its pipe's time
-// (66 clocks per warp-wide FMA) and a latency that a second warp per SM
-// sub-partition hides; FP32 is issue, at 1.1 (heat) and about 1.36 (KS) slots per
-// operation, above the latency of a level's shuffles and chain.
+// Estimated clocks per level of a block of `warps` warps with P points per thread
+// that owns its tile's points, from a fit to 2294 measured shapes (N from 2^10 to
+// 2^21; a clock is 1/2.07 us of event time, the SMs ran at 2.02 to 2.05 GHz): the
+// arithmetic of a level, the round through shared memory every L levels (170 to
+// 1000) and the exchange between blocks every L M levels (1450 and the polls of its
+// halo).  FP64 is its pipe's time (66 such clocks, 64 of the SM's, per warp-wide
+// FMA) and a latency that a second warp per SM sub-partition hides; the factors by
+// warps are the fit's too: one warp per sub-partition leaves 6 % of the pipe's slots
+// empty, three or four fill 2 % that two leave.  FP32 is issue, at 1.1 (heat) slots per
+// operation and for KS 1.36, or 1.5 where one warp per sub-partition has no other to
+// issue beside it, above the latency of a level's shuffles and chain.
 double level_clocks(int eq, int esize, int warps, int P, int L, int M, int h)
 {
     const double ops = eq == HEAT ? 3.0 : 7.0, w = warps / 4;

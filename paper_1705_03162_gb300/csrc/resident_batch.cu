@@ -16,6 +16,8 @@
 // slots: 256 heat and KS problems of 2^10..2^16 points, 2000 to 10000 steps, dataflow
 // launch 43.0 ms, this one 11.0.  FP64, for the batches that leave most of the chip
 // idle (resident_batch_choose), the levels' chains and exchanges.
+// A launch that the device refuses (too many blocks to hold at once) is the caller's
+// sign to run the dataflow form.
 #include <algorithm>
 #include <vector>
 

@@ -11,15 +11,17 @@
 // small; only the smallest grids, whose tiles do not fill the block's warps,
 // take more levels per exchange.
 //
-// What bounds it: the FP64 pipe.  A pass runs its rows of 32 cells on the SM's
-// four sub-partitions in turn, so its time goes with ceil(rows / 4); a grid of
-// 152 SMs x 128 cells or fewer has one row each, where the swept form took
-// 2H - 1 dependent levels per H levels of progress.  Clocks (2.07 GHz) per level
-// against the dataflow launch, Sod / limited everywhere: N = 4096 8100 / 8200
-// (21200 / 22600 when this form came), 65536 22500 / 32700 (28000 / 48700), 200000
-// 54000 / 91000 (62200 / 115100).  Grids whose cells do not fit shared memory (N above about
-// 330000), and Dirichlet ones above about 57000 cells (resident_euler_plan), keep that
-// launch.
+// What bounds it: the FP64 pipe (93 % busy with 200000 cells limited everywhere); on
+// small grids the chain of the passes and their barriers (Sod with 4096 cells: 5740
+// clocks per level in the tile, pipe 27 %) and, at an exchange, the wait for the
+// slowest tile.  A pass runs its rows of 32 cells on the SM's four sub-partitions in
+// turn, so its time goes with ceil(rows / 4); a grid of 152 SMs x 128 cells or fewer
+// has one row each, where the swept form took 2H - 1 dependent levels per H levels of
+// progress.  Clocks (1/2.07 us) per level, Sod in its first hundred steps / limited
+// everywhere, here (the dataflow launch when this form came): N = 4096 8100 / 8200
+// (21200 / 22600), 65536 22500 / 32700 (28000 / 48700), 200000 54000 / 91000 (62200 /
+// 115100).  Grids whose cells do not fit shared memory (N above about 330000), and
+// Dirichlet ones above about 57000 cells (resident_euler_plan), keep that launch.
 //
 // Dirichlet ends: the tile's slots beyond an end hold that end's ghost state in
 // both rows and are never updated (Appendix C's two ghost cells, and more of
@@ -46,8 +48,8 @@ constexpr int kThreads = SPLIT ? 256 : 512;
 // an interface, are tasks of their own on different warps (N = 4096: 8100 against
 // 10330 clocks per level).
 template <bool SPLIT>
-__global__ void __launch_bounds__(kThreads<SPLIT>) swept_resident_euler_kernel(const double* A, double* B, ResidentGeom g,
-                                                                        Coefs<double> cp)
+__global__ void __launch_bounds__(kThreads<SPLIT>)
+    swept_resident_euler_kernel(const double* A, double* B, ResidentGeom g, Coefs<double> cp)
 {
     using R = double;
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -11,7 +11,7 @@ namespace swp {
 
 // Two FP32 values advanced by one instruction (add / sub / fma .f32x2, each half
 // rounded as the scalar operation).  The FP32 pipe does the same operations per
-// clock either way, but a KS level's scalar FMAs, each reading three registers, took
+// clock either way (2.2 clocks per f32x2, 1.1 per scalar FMA), but a KS level's scalar FMAs, each reading three registers, took
 // 1.34 to 1.5 issue slots per operation where paired ones take 1.23 to 1.28: KS with
 // 2000003 points 1190 to 1087 clocks per level, 2^20 points 3 % faster, small grids
 // the same.  Heat's three operations do not pay for building the mixed pairs at a

@@ -53,10 +53,10 @@ template <> __device__ __forceinline__ Units<double> literal_units<double>() { r
 // FP64 sums, differences and products are written as fused multiply-adds:
 // a + b = fma(a, 1, b), a - b = fma(b, -1, a), a b = fma(a, b, -0), each rounded
 // once, with the same bits (signed zeros included).  GB300's FP64 unit takes a
-// warp-wide FMA whose three operands are vector registers every 68 clocks (at
-// 2.07 GHz, 152 SMs busy), but an add, a multiply, or an FMA with a literal,
-// constant-bank or uniform-register operand only every 80.6; every large FP64
-// path here is bound by that unit.  So the constants are kept in vector
+// warp-wide FMA whose three operands are vector registers every 64.0 clocks (the
+// SM's own clock counter, all 152 SMs busy, 1 to 4 warps per sub-partition), but an
+// add, a multiply, or an FMA with a literal, constant-bank or uniform-register operand
+// only every 76.0; every large FP64 path here is bound by that unit.  So the constants are kept in vector
 // registers whose value the compiler cannot see (Units).  Measured in G
 // point-updates/s before and after: KS 2^20 swept 39.8 / 42.5, classic graph
 // 29.6 / 33.6; heat 2^20 swept 169 / 188, 2^24 classic 169 / 195; Euler 2^20
