@@ -57,7 +57,11 @@ struct swp_problem {
     bool shape_known = false;
     ResidentShape shape;
     uint64_t* words = nullptr;
-    int* resident_status = nullptr;   // their status word: mapped host memory, so that reading it costs no copy
+    // their status word (nullptr before the first one): status_word, which costs no
+    // copy to look at, where the device uses the host's page tables (Grace); else
+    // device memory behind the words.  (A pinned word took 330 us of a problem's life.)
+    int* resident_status = nullptr;
+    int status_word = 0;
     uint32_t seq = 1;
 };
 
@@ -489,21 +493,20 @@ bool run_swept_resident(swp_problem* p, int64_t steps, swp_status* st)
     cudaError_t e = cudaSuccess;
     if (!p->words) {
         const RelaxedCapture relaxed;
-        if (!p->resident_status &&
-            cudaHostAlloc((void**)&p->resident_status, sizeof(int), cudaHostAllocMapped | cudaHostAllocPortable) !=
-                cudaSuccess) {
+        int shared = 0;
+        if (cudaDeviceGetAttribute(&shared, cudaDevAttrPageableMemoryAccessUsesHostPageTables, p->device) !=
+            cudaSuccess) {
             cudaGetLastError();
-            p->resident_status = nullptr;
-            return false;
+            shared = 0;
         }
-        *p->resident_status = 0;
-        e = cudaMalloc((void**)&p->words, bytes);
+        e = cudaMalloc((void**)&p->words, bytes + sizeof(int));
         if (e != cudaSuccess) {
             cudaGetLastError();
             p->words = nullptr;
             return false;
         }
-        e = cudaMemsetAsync(p->words, 0, bytes, p->stream);
+        p->resident_status = shared ? &p->status_word : (int*)((char*)p->words + bytes);
+        e = cudaMemsetAsync(p->words, 0, bytes + sizeof(int), p->stream);
         p->seq = 1;
     }
     const int64_t exchanges = resident_exchanges(p->shape, levels);
@@ -545,19 +548,22 @@ bool run_swept_resident(swp_problem* p, int64_t steps, swp_status* st)
 swp_status check_device_status(swp_problem* p)
 {
     bool gave_up = false;
-    if (p->status) {
-        int st = 0;
-        cudaError_t e = cudaMemcpy(&st, p->status, sizeof(int), cudaMemcpyDeviceToHost);
+    for (int* word : {p->status, p->resident_status}) {
+        if (!word) continue;
+        if (word == &p->status_word) {
+            volatile int* st = word;
+            if (*st != 0) {
+                *st = 0;
+                gave_up = true;
+            }
+            continue;
+        }
+        int st = 0;   // on the problem's own stream: other streams' work is not waited for
+        cudaError_t e = cudaMemcpyAsync(&st, word, sizeof(int), cudaMemcpyDeviceToHost, p->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(p->stream);
         if (e != cudaSuccess) return cuda_fail(e, "status read");
         if (st != 0) {
-            cudaMemset(p->status, 0, sizeof(int));
-            gave_up = true;
-        }
-    }
-    if (p->resident_status) {
-        volatile int* st = p->resident_status;
-        if (*st != 0) {
-            *st = 0;
+            cudaMemsetAsync(word, 0, sizeof(int), p->stream);
             gave_up = true;
         }
     }
@@ -960,7 +966,6 @@ swp_status swp_destroy(swp_problem* p)
     if (p->batch) swp_batch_destroy(p->batch);
     if (p->status) cudaFree(p->status);
     if (p->words) cudaFree(p->words);
-    if (p->resident_status) cudaFreeHost(p->resident_status);
     for (auto& g : p->graphs) cudaGraphExecDestroy(g.exec);
     if (p->capture_stream) cudaStreamDestroy(p->capture_stream);
     g_in_use -= p->bytes;

@@ -44,3 +44,44 @@ def test_default_advance_does_not_wait_for_other_streams(eq, bc, N, dtype):
         torch.cuda.synchronize()
         assert still and took < 0.2, took
         assert np.array_equal(got, want)
+
+
+def test_persistent_advance_does_not_wait_for_other_streams():
+    """The same for a launch whose status word is device memory."""
+    torch = pytest.importorskip("torch")
+    spec = spec_for("ks", "periodic", 4096)
+    u0 = state_for(spec)
+    with S.Problem(spec, u0, stream=torch.cuda.Stream()) as p:
+        for _ in range(2):
+            p.advance(10, "swept", 256, "persistent")
+            p.read()
+        torch.cuda.synchronize()
+        busy = torch.cuda.Event()
+        torch.cuda._sleep(1_000_000_000)
+        busy.record()
+        p.advance(10, "swept", 256, "persistent")
+        p.synchronize()
+        still = not busy.query()
+        torch.cuda.synchronize()
+        assert still
+
+
+def test_creating_and_closing_problems_costs_no_pinned_memory():
+    """A problem's life (create, a short default advance, read, close) takes no longer
+    than twice that of a problem that runs per-phase launches, which have no words:
+    a pinned allocation and its release alone take longer than the rest."""
+    spec = spec_for("heat", "periodic", 1024)
+    u0 = state_for(spec)
+
+    def life(n, launch):
+        took = []
+        for _ in range(60):
+            t0 = time.perf_counter()
+            with S.Problem(spec, u0) as p:
+                p.advance(10, "swept", n, launch)
+                p.read()
+            took.append(time.perf_counter() - t0)
+        return float(np.median(took[20:]))
+
+    life(0, "auto")
+    assert life(0, "auto") < 2 * life(128, "per_phase")
