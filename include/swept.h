@@ -100,7 +100,13 @@ typedef enum {
                                    330000 cells (Dirichlet ends: 57000);
                                    heat and KS in FP32 up to about
                                    2*10^6 points, and in tiles of the same
-                                   kind, a launch per some ten levels, above.
+                                   kind, a launch per some hundred levels,
+                                   above.
+                                   That launch is the fastest of one problem,
+                                   and spreads it over the chip: eight or more
+                                   small problems that advance at once go
+                                   faster as a batch, or on streams of their
+                                   own in the forms below, by name.
                                    Otherwise (wider FP64 grids, a stream under
                                    capture, a device that cannot hold that
                                    launch or its words): periodic heat
